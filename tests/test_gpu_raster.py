@@ -69,6 +69,36 @@ def test_posmaps_bit_exact(gc, H, W):
     assert valid[0].mean() > 0.1 and valid[1].mean() > 0.05 and valid[2, 0].all() and not valid[3].any()
 
 
+def _sized_mesh(kind, cam, rng):
+    """faces by the size of their pixel box: `tiny` mostly without a pixel centre, `mixed` from less than a pixel to
+    the whole view in one warp, `large` beyond the boxes that a warp concatenates, `bad` with vertices behind the
+    camera, at infinity and not a number"""
+    n, scale = {"tiny": (700, 0.02), "mixed": (200, 0.0), "large": (3, 3.0), "bad": (96, 0.5)}[kind]
+    size = np.full((n, 1, 1), scale) if scale else 10.0 ** rng.uniform(-3, 0.6, (n, 1, 1))
+    at = np.concatenate([rng.uniform(-0.7, 0.7, (n, 1, 2)), rng.uniform(2.0, 4.0, (n, 1, 1))], -1)
+    tri = at + size * rng.standard_normal((n, 3, 3)) * [1.0, 1.0, 0.1]
+    if kind == "large":  # fronto-parallel triangles that cover the view
+        tri = np.array([[[-9.0, -8.0, z], [9.0, -8.0, z], [0.0, 12.0, z + 0.2]] for z in (4.0, 3.0, 3.5)])
+    V = ((tri.reshape(-1, 3) - cam[9:12]) @ cam[:9].reshape(3, 3).astype(np.float64)).astype(np.float32)
+    if kind == "bad":
+        V[5], V[50, 1], V[90, 2], V[130] = np.inf, np.nan, -np.inf, 1e30
+        V[200] = V[201]  # a face of zero area
+    return V, np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("kind,H,W", [("tiny", 40, 56), ("mixed", 45, 70), ("large", 288, 331), ("bad", 33, 64)])
+def test_box_sizes_bit_exact(gc, kind, H, W):
+    cams = np.stack([synth.look_at_camera(az, 10.0, H, W) for az in (0.0, 25.0)])[None]
+    V, F = _sized_mesh(kind, cams[0, 0], np.random.default_rng(5))
+    pos, valid = gc.raster_posmaps(*_upload([(V, F)], cams), H, W)
+    torch.cuda.synchronize()
+    gc.device_status()
+    ref_p, ref_v = oracle.raster_views(V, F, cams[0], H, W)
+    np.testing.assert_array_equal(valid.cpu().numpy()[0], ref_v)
+    np.testing.assert_array_equal(pos.cpu().numpy()[0].view(np.uint32), ref_p.view(np.uint32))
+    assert ref_v.any()
+
+
 def test_posmaps_feed_the_correspondence_build(gc):
     # the rasterised maps of a blob are a valid input of the correspondence
     # build, which then gives the oracle's tables
