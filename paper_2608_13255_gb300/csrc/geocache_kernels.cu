@@ -65,6 +65,8 @@ __device__ __forceinline__ float fold_one(bool copy, float x0, float g, int n) {
 // texels (exact and order-free), the cluster combines the partial boxes through
 // distributed shared memory, and CTA 0 writes tau = tol_frac * sqrt(diag^2)
 // with the squares summed ((d0^2 + d1^2) + d2^2) in binary32.
+constexpr int kTauBlocks = 4;
+
 struct Box {
     float lo[3], hi[3];
     int any;
@@ -82,7 +84,7 @@ __device__ __forceinline__ void box_reduce_warp(Box& x) {
     }
 }
 
-__global__ void __launch_bounds__(256, 8) tau_kernel(const float* __restrict__ pos, const uint8_t* __restrict__ valid,
+__global__ void __launch_bounds__(256, kTauBlocks) tau_kernel(const float* __restrict__ pos, const uint8_t* __restrict__ valid,
                                                      int N, int HW, float tol_frac, int quads, float* __restrict__ tau) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -104,20 +106,31 @@ __global__ void __launch_bounds__(256, 8) tau_kernel(const float* __restrict__ p
         const size_t q0 = (size_t)rank * per, q1 = q0 + per < nq ? q0 + per : nq;
         const uint32_t* vq = reinterpret_cast<const uint32_t*>(valid + base);
         const float4* pq = reinterpret_cast<const float4*>(pos + 3 * base);
-#pragma unroll 4
-        for (size_t i = q0 + threadIdx.x; i < q1; i += blockDim.x) {
-            const uint32_t m = __ldg(vq + i);
-            if (!m) continue;  // background quads: their positions are not read
-            x.any = 1;
-            const float4 f0 = __ldg(pq + 3 * i), f1 = __ldg(pq + 3 * i + 1), f2 = __ldg(pq + 3 * i + 2);
-            const float f[12] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, f2.x, f2.y, f2.z, f2.w};
+        // four quads per thread and round: their validity words in flight
+        // together, then the positions of those with foreground (background
+        // quads' positions are not read)
+        for (size_t i0 = q0 + threadIdx.x; i0 < q1; i0 += 4 * blockDim.x) {
+            uint32_t m[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (!((m >> (8 * k)) & 0xffu)) continue;
+            for (int j = 0; j < 4; ++j) m[j] = i0 + j * blockDim.x < q1 ? __ldg(vq + i0 + j * blockDim.x) : 0u;
+            float4 f[4][3];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    x.lo[c] = fminf(x.lo[c], f[3 * k + c]);
-                    x.hi[c] = fmaxf(x.hi[c], f[3 * k + c]);
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    f[j][k] = m[j] ? __ldg(pq + 3 * (i0 + j * blockDim.x) + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float* p = reinterpret_cast<const float*>(f[j]);
+                x.any |= m[j] != 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (!((m[j] >> (8 * k)) & 0xffu)) continue;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        x.lo[c] = fminf(x.lo[c], p[3 * k + c]);
+                        x.hi[c] = fmaxf(x.hi[c], p[3 * k + c]);
+                    }
                 }
             }
         }
