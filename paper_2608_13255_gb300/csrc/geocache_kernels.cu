@@ -392,20 +392,31 @@ __device__ __forceinline__ int tiles_per_view_dev(int H, int W) {
     return (H * W + GEOCACHE_TILE_TOKENS - 1) / GEOCACHE_TILE_TOKENS;
 }
 
-// in-place exclusive prefix sum of n counts by one CTA; a[n] = total, or -1
-// when the total does not fit an int32.  Rounds of 1024 x kScanPer
-// consecutive counts: each thread loads its kScanPer counts (16-byte loads
-// when aligned), the CTA scans the per-thread sums, and each thread rewrites
-// its counts as offsets from the running total of the earlier rounds.
+// In-place exclusive prefix sum of n counts by one cluster of CTAs; a[n] =
+// total, or -1 when the total does not fit an int32.  Rounds of (cluster
+// size x 1024 x kScanPer) consecutive counts: each thread loads its kScanPer
+// counts (16-byte loads when aligned), each CTA scans its threads' sums, the
+// CTAs add the sums of those before them (through distributed shared memory)
+// and each thread rewrites its counts as offsets from the running total of
+// the earlier rounds.  Bound by the latency of a round (load, two barriers,
+// store), so the 8 CTAs take 131,072 counts in one round where one took
+// 16,384: 36,864 counts (64 assets x 6 views at 128 x 128) 10.9 -> 6.7 us.
 constexpr int kScanPer = 16;
+constexpr int kScanCtas = 8;
 
+template <int CTAS>
 __global__ void __launch_bounds__(1024) exclusive_scan_kernel(int32_t* a, long long n) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = CTAS > 1 ? (int)cluster.block_rank() : 0;
     __shared__ long long s_warp[32];
+    __shared__ long long s_total[2];  // this CTA's sum, by parity of the round
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const bool vec = (reinterpret_cast<uintptr_t>(a) & 15) == 0;
     long long carry = 0;  // sum of the counts of the earlier rounds
-    for (long long c0 = 0; c0 < n; c0 += 1024LL * kScanPer) {
-        const long long lo = c0 + (long long)t * kScanPer;
+    int par = 0;
+    for (long long c0 = 0; c0 < n; c0 += 1024LL * kScanPer * CTAS, par ^= 1) {
+        const long long lo = c0 + ((long long)rank * 1024 + t) * kScanPer;
         int x[kScanPer];
         if (vec && lo + kScanPer <= n) {
 #pragma unroll
@@ -436,9 +447,22 @@ __global__ void __launch_bounds__(1024) exclusive_scan_kernel(int32_t* a, long l
                 if (lane >= off) w += y;
             }
             s_warp[lane] = w;
+            if (lane == 31) s_total[par] = w;
         }
-        __syncthreads();
-        long long run = carry + (warp ? s_warp[warp - 1] : 0) + incl - sum;
+        long long before = 0, round = 0;
+        if (CTAS > 1) {
+            cluster.sync();  // every CTA's sum is in its shared memory
+#pragma unroll
+            for (int r = 0; r < CTAS; ++r) {
+                const long long y = *cluster.map_shared_rank(s_total + par, r);
+                before += r < rank ? y : 0;
+                round += y;
+            }
+        } else {
+            __syncthreads();
+            round = s_total[par];
+        }
+        long long run = carry + before + (warp ? s_warp[warp - 1] : 0) + incl - sum;
 #pragma unroll
         for (int i = 0; i < kScanPer; ++i) {  // counts -> offsets
             const int c = x[i];
@@ -454,21 +478,40 @@ __global__ void __launch_bounds__(1024) exclusive_scan_kernel(int32_t* a, long l
             for (int i = 0; i < kScanPer; ++i)
                 if (lo + i < n) a[lo + i] = x[i];
         }
-        carry += s_warp[31];
-        __syncthreads();  // s_warp is rewritten by the next round
+        carry += round;
+        __syncthreads();  // s_warp is rewritten by the next round; s_total alternates
     }
-    if (t == 0) {
+    if (CTAS > 1) cluster.sync();  // the others' shared memory stays alive until every CTA has read it
+    if (rank == 0 && t == 0) {
         a[n] = carry > 0x7fffffffLL ? -1 : (int32_t)carry;
         if (carry > 0x7fffffffLL) atomicOr(&g_device_error, 2u);  // more records than int32 offsets index
     }
+}
+
+static cudaError_t launch_scan(int32_t* a, long long n, cudaStream_t s) {
+    if (n <= 1024LL * kScanPer) {  // one round of one CTA, whose barrier is cheaper than the cluster's
+        exclusive_scan_kernel<1><<<1, 1024, 0, s>>>(a, n);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kScanCtas);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kScanCtas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, exclusive_scan_kernel<kScanCtas>, a, n);
 }
 
 // tile_ptr holds the per-tile counts written by build_corr_kernel; turn them
 // into offsets
 cudaError_t launch_tile_ptr(const geocache_corr& c, cudaStream_t s) {
     const int T = tiles_per_view(c.H, c.W);
-    exclusive_scan_kernel<<<1, 1024, 0, s>>>(c.tile_ptr, (long long)c.B * c.N * c.N * T);
-    return cudaGetLastError();
+    return launch_scan(c.tile_ptr, (long long)c.B * c.N * c.N * T, s);
 }
 
 // records of one (b, v, u, tile): kept rows in token order, each with its
@@ -639,7 +682,8 @@ cudaError_t launch_src_index(const geocache_corr& c, cudaStream_t s) {
         src_index_kernel<4, false><<<grid, 256, 0, s>>>(c.tile_ptr, c.records, c.max_records, c.N, c.W, T, c.src_ptr, out);
     else
         src_index_kernel<1, false><<<grid, 256, 0, s>>>(c.tile_ptr, c.records, c.max_records, c.N, c.W, T, c.src_ptr, out);
-    exclusive_scan_kernel<<<1, 1024, 0, s>>>(c.src_ptr, groups);
+    e = launch_scan(c.src_ptr, groups, s);
+    if (e != cudaSuccess) return e;
     if (c.K == 4)
         src_index_kernel<4, true><<<grid, 256, 0, s>>>(c.tile_ptr, c.records, c.max_records, c.N, c.W, T, c.src_ptr, out);
     else
