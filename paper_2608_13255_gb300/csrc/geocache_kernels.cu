@@ -514,7 +514,7 @@ cudaError_t launch_tile_ptr(const geocache_corr& c, cudaStream_t s) {
     return launch_scan(c.tile_ptr, (long long)c.B * c.N * c.N * T, s);
 }
 
-// records of one (b, v, u, tile): kept rows in token order, each with its
+// Records of one (b, v, u, tile): kept rows in token order, each with its
 // footprint's top-left tap and fractions (recomputed with the same device
 // functions as the tables, so the taps and weights they give are identical).
 // The tile's offsets and keep masks are loaded together, and the kept
@@ -527,7 +527,7 @@ cudaError_t launch_tile_ptr(const geocache_corr& c, cudaStream_t s) {
 // latency than the unbounded 43-register build (build graph of 128 assets:
 // 620 vs 641 us).
 template <int K>
-__global__ void __launch_bounds__(256, 8) fill_records_kernel(const float* __restrict__ pos,
+__global__ void __launch_bounds__(256, 8) fill_records_cta_kernel(const float* __restrict__ pos,
                                                            const geocache_camera* __restrict__ cams,
                                                            const uint8_t* __restrict__ keep,
                                                            const int32_t* __restrict__ tile_ptr, int N, int H,
@@ -621,15 +621,140 @@ __global__ void __launch_bounds__(256, 8) fill_records_kernel(const float* __res
     }
 }
 
-cudaError_t launch_fill_records(const geocache_corr& c, cudaStream_t s) {
+// The same for large builds, with one warp per tile: it reads the tile's masks
+// 4 tokens per lane and round, appends the kept ones (ranked by ballots) to a
+// list in shared memory and forms the records of a round (at most 128) with
+// their positions in flight together.  A tile without records costs a few
+// instructions, and no footprint runs in a partly filled warp but a tile's
+// last: what a round leaves below 32 waits for the next.
+//
+// 64 assets x 6 views at 128 x 128 (30,720 tiles of a pair): 48 -> 33.5 us.
+// The CTA per tile had 79% of its issue slots busy with the tiles' set-up (44 M
+// instructions against 18 M here); what bounds this one is the memory
+// latency of the dense tiles' rounds (42% of the slots busy), so small builds,
+// whose tiles all fit on the GPU at once, keep the CTA per tile: 480 tiles
+// 2.9 against 5.6 us, 7,680 tiles 14.2 against 16.2, 8,448 tiles (12 views)
+// 17.6 against 16.3.
+constexpr long long kFillWarpTiles = 8192;
+constexpr int kFillWarps = 4;  // per CTA: a CTA stays resident until its densest tile is done (8: 4 us slower)
+constexpr int kFillAhead = 4;  // positions in flight per lane
+
+template <int K>
+__global__ void __launch_bounds__(32 * kFillWarps) fill_records_kernel(const float* __restrict__ pos,
+                                                           const geocache_camera* __restrict__ cams,
+                                                           const uint8_t* __restrict__ keep,
+                                                           const int32_t* __restrict__ tile_ptr, int N, int H,
+                                                           int W, int T, geocache_tap_record* __restrict__ rec,
+                                                           long long max_records) {
+    constexpr int kRounds = GEOCACHE_TILE_TOKENS / 128;
+    __shared__ int s_list[kFillWarps][160];
+    __shared__ uint32_t s_mask[kFillWarps][kRounds][32];  // masks of tokens 128 k + 4 lane .. + 3, one byte each
+    __shared__ geocache_camera s_cam[kFillWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the asset's warps run over the tiles of its N (N - 1) off-diagonal pairs
+    // (diagonal pairs have no records): pair y has v = y / (N - 1), and u the
+    // (y mod (N - 1))-th view other than v
+    const int i_tile = (int)(blockIdx.x * kFillWarps + warp), b = blockIdx.y, y = i_tile / T;
+    if (y >= N * (N - 1)) return;
+    const int tile = i_tile - y * T, v = y / (N - 1), up = y - v * (N - 1);
+    const int u = up + (up >= v);
+    const int HW = H * W;
+    const size_t vu = (size_t)b * N * N + v * N + u;
+    const int r_first = __ldg(tile_ptr + vu * T + tile), r_next = __ldg(tile_ptr + vu * T + tile + 1);
+    // a tile without records has nothing to write; < 0: offsets overflowed (flagged by the scan)
+    if (r_next == r_first || r_first < 0) return;
+    const int p_base = tile * GEOCACHE_TILE_TOKENS;
+    const uint8_t* row = keep + vu * HW + p_base;
+    const bool words = (reinterpret_cast<uintptr_t>(row) & 3) == 0;
+#pragma unroll
+    for (int k = 0; k < kRounds; ++k) {
+        const int i = 128 * k + 4 * lane;
+        uint32_t m = 0;
+        if (words && p_base + i + 3 < HW) {
+            m = __ldg(reinterpret_cast<const uint32_t*>(row + i));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (p_base + i + e < HW) m |= (uint32_t)__ldg(row + i + e) << (8 * e);
+        }
+        s_mask[warp][k][lane] = m;
+    }
+    if (lane < 16)
+        reinterpret_cast<float*>(s_cam + warp)[lane] = __ldg(reinterpret_cast<const float*>(cams + (size_t)b * N + u) + lane);
+    int* list = s_list[warp];
+    const float* pos_v = pos + 3 * ((size_t)b * N + v) * HW;
+    const uint32_t below = (1u << lane) - 1u;
+    long long r = r_first;  // record of list[0]
+    int listed = 0;
+#pragma unroll 1
+    for (int k = 0; k < kRounds; ++k) {
+        const uint32_t m = s_mask[warp][k][lane];
+        const bool last = k == kRounds - 1;
+        if (!__any_sync(0xffffffffu, m) && !last) continue;
+        int at = listed;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t kept = __ballot_sync(0xffffffffu, (m >> (8 * e)) & 0xffu);
+            at += __popc(kept & below);
+            listed += __popc(kept);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t mask = (m >> (8 * e)) & 0xffu;
+            if (mask) list[at++] = (p_base + 128 * k + 4 * lane + e) | (int)(mask << 28);
+        }
+        __syncwarp();
+        const int n = last ? listed : listed & ~31;
+#pragma unroll 1
+        for (int j0 = 0; j0 < n; j0 += 32 * kFillAhead) {
+            int tm[kFillAhead];
+            float X[kFillAhead][3];
+#pragma unroll
+            for (int g = 0; g < kFillAhead; ++g) {
+                const int j = j0 + 32 * g + lane;
+                tm[g] = list[j < n ? j : 0];
+                const float* x = pos_v + 3 * (size_t)(tm[g] & 0x0fffffff);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) X[g][c] = j < n ? __ldg(x + c) : 0.0f;
+            }
+#pragma unroll
+            for (int g = 0; g < kFillAhead; ++g) {
+                const int j = j0 + 32 * g + lane;
+                if (j >= n) break;
+                Footprint f;
+                footprint<K>(s_cam[warp], X[g][0], X[g][1], X[g][2], H, W, f);
+                if (r + j < max_records)
+                    reinterpret_cast<int4*>(rec)[r + j] =
+                        make_int4(tm[g], f.j0 * W + f.i0, __float_as_int(K == 4 ? f.ax[1] : 0.0f),
+                                  __float_as_int(K == 4 ? f.ay[1] : 0.0f));
+                else
+                    atomicOr(&g_device_error, 2u);  // records beyond the capacity are dropped
+            }
+        }
+        int rest = 0;
+        if (n + lane < listed) rest = list[n + lane];
+        __syncwarp();
+        if (n + lane < listed) list[lane] = rest;
+        r += n;
+        listed -= n;
+    }
+}
+
+template <int K>
+static void launch_fill_records_k(const geocache_corr& c, cudaStream_t s) {
     const int T = tiles_per_view(c.H, c.W);
-    dim3 grid(T, c.N * (c.N - 1), c.B);
-    if (c.K == 4)
-        fill_records_kernel<4><<<grid, 256, 0, s>>>(c.pos, c.cams, c.keep, c.tile_ptr, c.N, c.H, c.W, T, c.records,
-                                                    c.max_records);
+    const long long tiles = (long long)T * c.N * (c.N - 1);  // per asset
+    if (tiles * c.B >= kFillWarpTiles)
+        fill_records_kernel<K><<<dim3((unsigned)((tiles + kFillWarps - 1) / kFillWarps), c.B), 32 * kFillWarps, 0, s>>>(
+            c.pos, c.cams, c.keep, c.tile_ptr, c.N, c.H, c.W, T, c.records, c.max_records);
     else
-        fill_records_kernel<1><<<grid, 256, 0, s>>>(c.pos, c.cams, c.keep, c.tile_ptr, c.N, c.H, c.W, T, c.records,
-                                                    c.max_records);
+        fill_records_cta_kernel<K><<<dim3(T, c.N * (c.N - 1), c.B), 256, 0, s>>>(
+            c.pos, c.cams, c.keep, c.tile_ptr, c.N, c.H, c.W, T, c.records, c.max_records);
+}
+
+cudaError_t launch_fill_records(const geocache_corr& c, cudaStream_t s) {
+    if (c.K == 4) launch_fill_records_k<4>(c, s);
+    else launch_fill_records_k<1>(c, s);
     return cudaGetLastError();
 }
 
