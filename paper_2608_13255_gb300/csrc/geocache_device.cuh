@@ -30,9 +30,10 @@ __device__ __forceinline__ void taps_clear(Taps& t) {
 }
 
 // x_c = R X + t with each row summed ((R0 X0 + R1 X1) + R2 X2) + t, then the
-// pinhole projection.  Returns false when the point is not in front.
+// pinhole projection (depth receives the camera z).  Returns false when the
+// point is not in front.
 __device__ __forceinline__ bool project(const geocache_camera& c, float X0, float X1, float X2,
-                                        float& uu, float& vv) {
+                                        float& uu, float& vv, float& depth) {
     float xc[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -41,6 +42,7 @@ __device__ __forceinline__ bool project(const geocache_camera& c, float X0, floa
         s = __fadd_rn(s, __fmul_rn(c.R[3 * r + 2], X2));
         xc[r] = __fadd_rn(s, c.t[r]);
     }
+    depth = xc[2];
     if (!(xc[2] > 0.0f)) return false;
     uu = __fadd_rn(__fmul_rn(c.fx, __fdiv_rn(xc[0], xc[2])), c.cx);
     vv = __fadd_rn(__fmul_rn(c.fy, __fdiv_rn(xc[1], xc[2])), c.cy);
@@ -65,9 +67,9 @@ struct Footprint {
 
 template <int K>
 __device__ __forceinline__ bool footprint(const geocache_camera& cam, float X0, float X1, float X2, int H, int W,
-                                          Footprint& f) {
+                                          Footprint& f, float& depth) {
     float uu, vv;
-    if (!project(cam, X0, X1, X2, uu, vv)) return false;
+    if (!project(cam, X0, X1, X2, uu, vv, depth)) return false;
     if (K == 1) {
         if (!(uu >= 0.0f && uu < (float)W && vv >= 0.0f && vv < (float)H)) return false;
         f.i0 = (int)floorf(uu);
@@ -86,6 +88,13 @@ __device__ __forceinline__ bool footprint(const geocache_camera& cam, float X0, 
     f.ay[0] = __fsub_rn(1.0f, fy);
     f.ay[1] = fy;
     return true;
+}
+
+template <int K>
+__device__ __forceinline__ bool footprint(const geocache_camera& cam, float X0, float X1, float X2, int H, int W,
+                                          Footprint& f) {
+    float depth;
+    return footprint<K>(cam, X0, X1, X2, H, W, f, depth);
 }
 
 // Per-tap tests: inside the image, non-zero weight factors, foreground

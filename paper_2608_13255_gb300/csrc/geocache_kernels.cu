@@ -227,7 +227,7 @@ static_assert(GEOCACHE_TILE_TOKENS % kBuildThreads == 0, "a build CTA's tokens l
 // or 4): its foreground tokens are compacted across the slices and each
 // thread takes up to REP of them in turn, so that fewer lanes idle through
 // the source loop (the background is ~60% of a view).  REP = 4 for large
-// builds (128 batch128 assets: 504 -> 465 us for the build graph), 1 for
+// builds with tables (large builds without take build_keep_kernel), 1 for
 // small ones, where the 4x fewer CTAs would not fill the GPU.
 template <int K, bool TABLES, int REP>
 __global__ void __launch_bounds__(kBuildThreads) build_corr_kernel(const float* __restrict__ pos,
@@ -344,36 +344,299 @@ __global__ void __launch_bounds__(kBuildThreads) build_corr_kernel(const float* 
     }
 }
 
-template <int REP>
+// ---- large builds without tables: keep masks with an occlusion test first --
+// Most (token, source view) pairs keep no tap because the token's point X is
+// hidden in the source view: the surface there is nearer than X by more than
+// the tolerance.  source_depth_kernel therefore stores, for each block of 8 x 8
+// texels of every view, a camera depth that no kept tap's target exceeds, and
+// build_keep_kernel tests taps only for the pairs that pass (17% of the pairs
+// of a 6-view batch keep a tap, 25% pass; with blocks of 4 and 16: 23%, 28%).
+//
+// The bound: a kept tap's texel P lies within tau of X (to 1e-6 relative in
+// binary32), so the depths z = R2 . x + t2 of P and X differ by at most
+// |R2| tau, plus the rounding of both, at most 4 * 2^-24 S each with
+// S = |R2| . |x| + |t2| summed by component.  A block's value is the largest
+// z + 1e-6 S of its foreground texels plus |R2| tau (1 + 1e-5) and the change of
+// S over a distance tau; -inf without foreground.  It covers 9 x 9 texels: the
+// block and the column and row after it, so that one value serves every
+// footprint whose top-left tap lies in the block.  A NaN never rejects.
+//
+// The values lie in the keep masks' diagonal rows (u = v), which hold no masks
+// and are cleared after the build, so that no scratch is needed.
+constexpr int kDepthBlock = 8;
+__host__ __device__ inline int depth_blocks(int n) { return (n + kDepthBlock - 1) / kDepthBlock; }
+
+__device__ __forceinline__ float* depth_row(uint8_t* keep, size_t view, int v, int N, size_t HW) {
+    const uintptr_t p = reinterpret_cast<uintptr_t>(keep + (view * N + v) * HW);
+    return reinterpret_cast<float*>((p + 3) & ~(uintptr_t)3);
+}
+
+// the 16-byte chunk `i` of the address range [p, p + n), cleared; i runs from 0
+// to n / 16 + 1 (an unaligned range has a part of a chunk at either end)
+__device__ __forceinline__ void clear_chunk(uint8_t* p, int n, int i) {
+    const intptr_t lo = 16 * (intptr_t)i - (reinterpret_cast<uintptr_t>(p) & 15);
+    if (lo >= 0 && lo + 16 <= n) {
+        *reinterpret_cast<uint4*>(p + lo) = make_uint4(0, 0, 0, 0);
+    } else {
+        for (intptr_t k = lo < 0 ? 0 : lo; k < lo + 16 && k < n; ++k) p[k] = 0;
+    }
+}
+
+// One warp per 4 blocks of a row of blocks: lane l reads column l of their 9
+// texel rows (coalesced; a warp per block, 9 texels a row, took 27 us against
+// 15 at 64 assets x 6 views of 128 x 128, bound by the L1's wavefronts), and 9
+// lanes the column after them.
+__global__ void __launch_bounds__(256) source_depth_kernel(const float* __restrict__ pos,
+                                                           const uint8_t* __restrict__ valid,
+                                                           const geocache_camera* __restrict__ cams,
+                                                           const float* __restrict__ tau, int N, int H, int W,
+                                                           uint8_t* keep) {
+    constexpr int kRows = kDepthBlock + 1;
+    const int nbx = depth_blocks(W), n_strips = (nbx + 3) / 4;
+    const int lane = threadIdx.x & 31, strip = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (strip >= n_strips * depth_blocks(H)) return;
+    const int v = blockIdx.y, b = blockIdx.z;
+    const size_t view = (size_t)b * N + v, HW = (size_t)H * W;
+    const float* cam = reinterpret_cast<const float*>(cams + view);
+    const float r0 = __ldg(cam + 6), r1 = __ldg(cam + 7), r2 = __ldg(cam + 8), t2 = __ldg(cam + 11);
+    const int by = strip / n_strips, y0 = by * kDepthBlock, x0 = (strip - by * n_strips) * 4 * kDepthBlock;
+    const uint8_t* valid_v = valid + view * HW;
+    const float* pos_v = pos + 3 * view * HW;
+    bool fg[kRows + 1];
+    float p[kRows + 1][3];
+#pragma unroll
+    for (int k = 0; k <= kRows; ++k) {  // the last round: lane l's texel is row l of the next strip's first column
+        const int y = k < kRows ? y0 + k : y0 + lane, x = k < kRows ? x0 + lane : x0 + 4 * kDepthBlock;
+        const size_t q = (size_t)y * W + x;
+        fg[k] = y < H && x < W && (k < kRows || lane < kRows);
+        fg[k] = fg[k] && __ldg(valid_v + q);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) p[k][c] = fg[k] ? __ldg(pos_v + 3 * q + c) : 0.0f;
+    }
+    float z = -INFINITY, z_next = -INFINITY;
+#pragma unroll
+    for (int k = 0; k <= kRows; ++k) {
+        const float s = fabsf(r0 * p[k][0]) + fabsf(r1 * p[k][1]) + fabsf(r2 * p[k][2]) + fabsf(t2);
+        float far = r0 * p[k][0] + r1 * p[k][1] + r2 * p[k][2] + t2 + 1e-6f * s;
+        far = far <= FLT_MAX ? far : INFINITY;  // an overflow or NaN: the block rejects nothing
+        if (fg[k]) (k < kRows ? z : z_next) = fmaxf(k < kRows ? z : z_next, far);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) z_next = fmaxf(z_next, __shfl_xor_sync(0xffffffffu, z_next, off));
+    float block = z;  // over the block's 8 columns, then the next block's first
+#pragma unroll
+    for (int off = 1; off < kDepthBlock; off <<= 1) block = fmaxf(block, __shfl_xor_sync(0xffffffffu, block, off));
+    const float after = __shfl_down_sync(0xffffffffu, z, kDepthBlock);
+    block = fmaxf(block, lane < 32 - kDepthBlock ? after : z_next);
+    const int bx = (x0 + lane) / kDepthBlock;
+    if (lane % kDepthBlock == 0 && bx < nbx) {
+        const float t = __ldg(tau + b);
+        const float norm2 = sqrtf(r0 * r0 + r1 * r1 + r2 * r2), norm1 = fabsf(r0) + fabsf(r1) + fabsf(r2);
+        depth_row(keep, view, v, N, HW)[by * nbx + bx] = block + t * (1.00001f * norm2 + 1e-6f * norm1);
+    }
+}
+
+// One CTA per tile (asset b, target view v, GEOCACHE_TILE_TOKENS tokens).  Its
+// foreground tokens are compacted with their positions; each thread then
+// projects a token into every source view, and the pairs that pass the depth
+// test are queued per warp and their taps tested 32 at a time, so that the
+// gathers of a warp are full.  The tile's rows of the masks are cleared first
+// and only kept masks written; the CTA's counts are the tile's.
+//
+// 64 assets x 6 views at 128 x 128: 140 -> 87 us (and 15 us for the depths).
+// With the taps of every pair tested (16 scalar gathers each) the L1's
+// wavefronts were 71% and the issue slots 67% busy; here the slots are 78% busy
+// with the projections (78 M instructions against 105 M), the wavefronts 56%.
+// 6 resident CTAs per SM (40 registers); 7 or 8 spill and take 116 us.
+struct PairQueue {
+    uint32_t what[64];  // compacted token | source view << 10 | taps of weight 0 << 16
+    uint32_t at[64];    // footprint corner: (i0 + 1) | (j0 + 1) << 16
+};
+
+template <int K>
+__global__ void __launch_bounds__(kBuildThreads) build_keep_kernel(const float* __restrict__ pos,
+                                                                   const uint8_t* __restrict__ valid,
+                                                                   const geocache_camera* __restrict__ cams,
+                                                                   const float* __restrict__ tau, int N, int H, int W,
+                                                                   uint8_t* keep, int32_t* __restrict__ tile_cnt) {
+    constexpr int kReps = GEOCACHE_TILE_TOKENS / kBuildThreads, kWarps = kBuildThreads / 32;
+    __shared__ geocache_camera s_cam[GEOCACHE_MAX_VIEWS];
+    __shared__ float4 s_tok[GEOCACHE_TILE_TOKENS];  // foreground tokens: position, token
+    __shared__ PairQueue s_queue[kWarps];
+    __shared__ int s_wcnt[kReps][kWarps];
+    __shared__ int s_cnt[GEOCACHE_MAX_VIEWS];
+    const int HW = H * W, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int p_base = blockIdx.x * GEOCACHE_TILE_TOKENS, v = blockIdx.y, b = blockIdx.z;
+    const int n_tok = min(GEOCACHE_TILE_TOKENS, HW - p_base);
+    for (int i = t; i < N * 16; i += kBuildThreads)
+        reinterpret_cast<float*>(s_cam)[i] = __ldg(reinterpret_cast<const float*>(cams + (size_t)b * N) + i);
+    if (t < N) s_cnt[t] = 0;
+    const size_t view = (size_t)b * N + v, view0 = view * HW;
+    // compaction of the foreground tokens, in token order
+    unsigned bal[kReps];
+    bool fg[kReps];
+#pragma unroll
+    for (int h = 0; h < kReps; ++h) {
+        const int i = h * kBuildThreads + t;
+        fg[h] = i < n_tok && __ldg(valid + view0 + p_base + i);
+        bal[h] = __ballot_sync(0xffffffffu, fg[h]);
+        if (lane == 0) s_wcnt[h][warp] = __popc(bal[h]);
+    }
+    // the tile's mask rows of the other views, cleared
+    uint8_t* const rows = keep + view * N * HW + p_base;
+    if (((reinterpret_cast<uintptr_t>(rows) | (uintptr_t)HW | (uintptr_t)n_tok) & 15) == 0) {
+        for (int i = t; i < N * 64; i += kBuildThreads) {
+            const int u = i >> 6, c = i & 63;
+            if (u != v && 16 * c < n_tok) reinterpret_cast<uint4*>(rows + (size_t)u * HW)[c] = make_uint4(0, 0, 0, 0);
+        }
+    } else {
+        for (int i = t; i < N * 128; i += kBuildThreads) {  // at most 65 chunks a row
+            const int u = i >> 7, c = i & 127;
+            if (u != v && c <= n_tok / 16 + 1) clear_chunk(rows + (size_t)u * HW, n_tok, c);
+        }
+    }
+    __syncthreads();
+    int n_fg = 0;
+#pragma unroll
+    for (int h = 0; h < kReps; ++h) {
+        int before = n_fg, tot = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            before += w < warp ? s_wcnt[h][w] : 0;
+            tot += s_wcnt[h][w];
+        }
+        if (fg[h]) {
+            const int p = p_base + h * kBuildThreads + t;
+            const float* q = pos + 3 * (view0 + p);
+            s_tok[before + __popc(bal[h] & ((1u << lane) - 1u))] =
+                make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __int_as_float(p));
+        }
+        n_fg += tot;
+    }
+    __syncthreads();
+    const float tu = __ldg(tau + b), tau2 = __fmul_rn(tu, tu);
+    const int nbx = depth_blocks(W);
+    PairQueue& q = s_queue[warp];
+    const uint32_t below = (1u << lane) - 1u;
+    int head = 0, queued = 0;
+    auto test_taps = [&]() {  // the queue's pair `head + lane`
+        const uint32_t what = q.what[(head + lane) & 63], at = q.at[(head + lane) & 63];
+        const int u = (int)((what >> 10) & 63u), i0 = (int)(at & 0xffffu) - 1, j0 = (int)(at >> 16) - 1;
+        const float4 X = s_tok[what & 1023u];
+        const uint8_t* valid_u = valid + ((size_t)b * N + u) * HW;
+        const float* pos_u = pos + 3 * ((size_t)b * N + u) * HW;
+        int mask = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int col = i0 + (k & 1), row = j0 + (k >> 1);
+            if ((unsigned)col >= (unsigned)W || (unsigned)row >= (unsigned)H || ((what >> (16 + k)) & 1u)) continue;
+            const int tap = row * W + col;
+            const int ok = __ldg(valid_u + tap) != 0;
+            const int near = sqdist(pos_u + 3 * (size_t)tap, X.x, X.y, X.z) <= tau2;
+            mask |= (ok & near) << k;
+        }
+        if (mask) {
+            keep[(view * N + u) * HW + __float_as_int(X.w)] = (uint8_t)mask;
+            atomicAdd(&s_cnt[u], 1);
+        }
+    };
+#pragma unroll 1
+    for (int j0 = 0; j0 < n_fg; j0 += kBuildThreads) {
+        const int j = j0 + t;
+        const bool work = j < n_fg;
+        const float4 X = s_tok[work ? j : 0];
+        for (int u = 0; u < N; ++u) {
+            if (u == v) continue;
+            bool pass = false;
+            uint32_t what = 0, at = 0;
+            Footprint f;
+            float depth;
+            if (work && footprint<K>(s_cam[u], X.x, X.y, X.z, H, W, f, depth)) {
+                const float* far = depth_row(keep, (size_t)b * N + u, u, N, HW);
+                const int blk = max(f.j0, 0) / kDepthBlock * nbx + max(f.i0, 0) / kDepthBlock;
+                pass = !(depth > far[blk]);
+                uint32_t dead = 0;  // taps of weight 0
+                if (K == 4)
+                    dead = (f.ax[0] == 0.0f ? 5u : 0u) | (f.ax[1] == 0.0f ? 10u : 0u) | (f.ay[0] == 0.0f ? 3u : 0u) |
+                           (f.ay[1] == 0.0f ? 12u : 0u);
+                what = (uint32_t)j | ((uint32_t)u << 10) | (dead << 16);
+                at = (uint32_t)(f.i0 + 1) | ((uint32_t)(f.j0 + 1) << 16);
+            }
+            const uint32_t passed = __ballot_sync(0xffffffffu, pass);
+            if (pass) {
+                const int e = (head + queued + __popc(passed & below)) & 63;
+                q.what[e] = what;
+                q.at[e] = at;
+            }
+            queued += __popc(passed);
+            if (queued >= 32) {
+                __syncwarp();
+                test_taps();
+                __syncwarp();  // its entries are rewritten by later pairs
+                head += 32;
+                queued -= 32;
+            }
+        }
+    }
+    __syncwarp();
+    if (lane < queued) test_taps();
+    if (tile_cnt) {
+        __syncthreads();
+        if (t < N) tile_cnt[(view * N + t) * gridDim.x + blockIdx.x] = s_cnt[t];
+    }
+}
+
+// the diagonal rows, cleared of the depths
+__global__ void __launch_bounds__(256) clear_diagonal_kernel(uint8_t* keep, int N, int HW) {
+    uint8_t* row = keep + ((size_t)blockIdx.z * N + blockIdx.y) * N * HW + (size_t)blockIdx.y * HW;
+    clear_chunk(row, HW, blockIdx.x * 256 + threadIdx.x);
+}
+
+template <int K, bool TABLES, int REP>
 static void launch_build_corr_rep(const geocache_corr& c, int32_t* cnt, cudaStream_t s) {
     const int HW = c.H * c.W;
     const dim3 grid((HW + kBuildThreads * REP - 1) / (kBuildThreads * REP), c.N, c.B);
-    if (c.K == 4 && c.idx)
-        build_corr_kernel<4, true, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W,
-                                                                       c.idx, c.w, c.keep, cnt);
-    else if (c.K == 4)
-        build_corr_kernel<4, false, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W,
-                                                                        c.idx, c.w, c.keep, cnt);
-    else if (c.idx)
-        build_corr_kernel<1, true, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W,
-                                                                       c.idx, c.w, c.keep, cnt);
-    else
-        build_corr_kernel<1, false, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W,
-                                                                        c.idx, c.w, c.keep, cnt);
+    build_corr_kernel<K, TABLES, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx,
+                                                                     c.w, c.keep, cnt);
 }
 
+// Tiles from which the depth test pays for its two extra launches and its
+// fewer, larger CTAs (masks of 6 or 12 views at 128 x 128, old and new: 384
+// tiles 18.3 and 20.6 us, 768 tiles 27.7 and 25.3, 768 (12 views) 59.6 and 49.1,
+// 6,144 tiles 142 and 104; 600 tiles of 61 x 97: 17.2 and 17.4).
+constexpr long long kDepthTestTiles = 700;
+
 cudaError_t launch_build_corr(const geocache_corr& c, cudaStream_t s) {
+    const int HW = c.H * c.W, T = tiles_per_view(c.H, c.W);
+    const long long tiles = (long long)T * c.N * c.B;
+    const long long nb = (long long)depth_blocks(c.H) * depth_blocks(c.W);
+    // the depths of a view fit its diagonal row (with 3 bytes to align them)
+    if (!c.idx && c.keep && tiles >= kDepthTestTiles && 4 * nb + 3 <= HW) {
+        const long long strips = (long long)((depth_blocks(c.W) + 3) / 4) * depth_blocks(c.H);
+        source_depth_kernel<<<dim3((unsigned)((strips + 7) / 8), c.N, c.B), 256, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N,
+                                                                                   c.H, c.W, c.keep);
+        if (c.K == 4)
+            build_keep_kernel<4><<<dim3(T, c.N, c.B), kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H,
+                                                                             c.W, c.keep, c.tile_ptr);
+        else
+            build_keep_kernel<1><<<dim3(T, c.N, c.B), kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H,
+                                                                             c.W, c.keep, c.tile_ptr);
+        clear_diagonal_kernel<<<dim3((unsigned)(HW / 4096 + 1), c.N, c.B), 256, 0, s>>>(c.keep, c.N, HW);
+        return cudaGetLastError();
+    }
     int32_t* cnt = nullptr;
     if (c.tile_ptr) {
-        const size_t n = (size_t)c.B * c.N * c.N * tiles_per_view(c.H, c.W) + 1;
+        const size_t n = (size_t)c.B * c.N * c.N * T + 1;
         cudaError_t e = cudaMemsetAsync(c.tile_ptr, 0, n * sizeof(int32_t), s);
         if (e != cudaSuccess) return e;
         cnt = c.tile_ptr;
     }
-    // 4 slices per CTA once the build has at least 4096 CTAs of 1024 tokens
-    const long long ctas4 = (long long)tiles_per_view(c.H, c.W) * c.N * c.B;
-    if (ctas4 >= 4096) launch_build_corr_rep<4>(c, cnt, s);
-    else launch_build_corr_rep<1>(c, cnt, s);
+    if (!c.idx)
+        c.K == 4 ? launch_build_corr_rep<4, false, 1>(c, cnt, s) : launch_build_corr_rep<1, false, 1>(c, cnt, s);
+    else if (tiles >= 4096)  // 4 slices per CTA once the build has at least 4096 CTAs of 1024 tokens
+        c.K == 4 ? launch_build_corr_rep<4, true, 4>(c, cnt, s) : launch_build_corr_rep<1, true, 4>(c, cnt, s);
+    else
+        c.K == 4 ? launch_build_corr_rep<4, true, 1>(c, cnt, s) : launch_build_corr_rep<1, true, 1>(c, cnt, s);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,50 @@ def test_tables_bit_exact_k1(gc, workloads, name):
     _compare_tables(w, g, 1)
 
 
+@pytest.mark.parametrize("H,W,B,K,scene", [(24, 21, 320, 4, "plain"), (24, 21, 320, 1, "plain"), (37, 29, 160, 4, "far"),
+                                           (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd")])
+def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
+    # builds of at least 700 tiles test a source depth before the taps, and fill their records with a warp per tile
+    # from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
+    # that the oracle checks).  far: an asset 3,000 units from the origin (the depths' rounding); scaled: cameras with
+    # rows of other lengths than 1; odd: infinite, huge and NaN positions, and an empty asset
+    w = synth.make_workload("batch128", B=6, H=H, W=W)
+    w.pos, w.cams = w.pos.copy(), w.cams.copy()
+    R, t = w.cams[..., :9].reshape(6, w.N, 3, 3), w.cams[..., 9:12]
+    if scene == "far":
+        shift = np.array([3000.0, -1500.0, 800.0])
+        w.cams[..., 9:12] = t - (R.astype(np.float64) @ shift)
+        w.pos = (w.pos.astype(np.float64) + shift).astype(np.float32)
+    if scene == "scaled":
+        w.cams[..., :12] *= np.float32(3.7)
+    if scene == "odd":
+        fg = np.argwhere(w.valid[:3] > 0)
+        for k, x in enumerate((np.inf, 3e38, np.nan, 1e20, -np.inf)):
+            w.pos[tuple(fg[7 + 31 * k])][k % 3] = x
+        w.valid[4] = 0
+    big = synth.replicate_assets(w, B)
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    c = gc.build_sparse_corr(d(big.pos), d(big.valid), d(big.cams), K=K)
+    keep = torch.full((B, w.N, w.N, H, W), 77, dtype=torch.uint8, device="cuda")
+    gc.build_corr(gc.make_corr(d(big.pos), d(big.valid), d(big.cams), torch.zeros(B, device="cuda"), K=K, keep=keep))
+    whole = gc.build_corr(c)  # masks, offsets and records in one call
+    gc.device_status()
+    assert torch.equal(keep, c.keep)
+    T, pairs = gc.tiles_per_view(H, W), w.N * w.N
+    ptr, rec = whole._keep["tile_ptr"], whole._keep["records"]
+    n_rec = 0
+    for b in range(6):
+        one = gc.build_sparse_corr(d(w.pos[b:b + 1]), d(w.valid[b:b + 1]), d(w.cams[b:b + 1]), K=K)
+        p1, r1 = one._keep["tile_ptr"], one._keep["records"]
+        for k in range(b, B, 6):
+            off = ptr[k * pairs * T:(k + 1) * pairs * T + 1]
+            assert torch.equal(c.keep[k], one.keep[0])
+            assert torch.equal(off - off[0], p1)
+            assert torch.equal(rec[int(off[0]):int(off[-1])], r1[:int(p1[-1])])
+        n_rec += int(p1[-1])
+    assert n_rec > 100
+
+
 def _run_step(gc, w, g, anchors, params, pred=None, mode="sparse", inplace=False, xinplace=False,
               seed_extra=0, C=None, minimal_ws=False):
     """One cached step on the GPU and in the oracle from the same inputs."""
