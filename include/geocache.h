@@ -199,10 +199,22 @@ int geocache_build_corr(geocache_corr* corr, void* stream);
  * kept (target token, source view) rows of every G_{u->v}): builds tau, the
  * keep masks and tile_ptr (corr->keep and corr->tile_ptr are required), then
  * synchronises `stream` and returns the count in *count.  Allocate
- * max_records >= *count records and call geocache_build_corr to fill them.
+ * max_records >= *count records and call geocache_fill_records (or
+ * geocache_build_corr, which also builds the rest again) to fill them.
  * Returns GEOCACHE_OK, EINVAL, ESHAPE, ECUDA.
  * ------------------------------------------------------------------------ */
 int geocache_corr_record_count(geocache_corr* corr, int64_t* count, void* stream);
+
+/* --------------------------------------------------------------------------
+ * geocache_fill_records -- the last part of geocache_build_corr (Sec. 3.2,
+ * "Correspondence operator"): writes corr->records (and src_ptr / src_rec when
+ * given) from the keep masks and tile_ptr that geocache_corr_record_count or
+ * geocache_build_corr wrote for the same pos, valid, cams, sizes and K; tau
+ * and the tables are not touched.  Same records and same handling of
+ * max_records as geocache_build_corr.  Asynchronous.
+ * Returns GEOCACHE_OK, EINVAL, ESHAPE, EALIAS, ECUDA.
+ * ------------------------------------------------------------------------ */
+int geocache_fill_records(geocache_corr* corr, void* stream);
 
 /* --------------------------------------------------------------------------
  * geocache_transport_workspace -- number of floats of workspace to give

@@ -99,52 +99,8 @@ int read_total(const geocache_corr* c, int64_t* total, cudaStream_t s) {
     return GEOCACHE_OK;
 }
 
-}  // namespace
-
-int geocache::set_error(int status, const char* fmt, ...) {
-    char buf[512];
-    va_list ap;
-    va_start(ap, fmt);
-    vsnprintf(buf, sizeof buf, fmt, ap);
-    va_end(ap);
-    g_last_error = buf;
-    return status;
-}
-
-extern "C" {
-
-int geocache_abi_version(void) { return GEOCACHE_ABI_VERSION; }
-
-int geocache_device_status(void* stream) {
-    unsigned int word = 0, raster_word = 0;
-    cudaError_t e = geocache::read_device_error(&word, true, (cudaStream_t)stream);
-    if (e == cudaSuccess) e = geocache::read_raster_error(&raster_word, true, (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(e, "reading the device status word");
-    word |= raster_word;
-    if (word & 2u)
-        return fail(GEOCACHE_ESHAPE, "a sparse-form build had more records than max_records (status word 0x%x); "
-                                     "query geocache_corr_record_count and rebuild", word);
-    if (word & 4u)
-        return fail(GEOCACHE_EINVAL, "a record permutation entry was outside [0, max_records) (status word 0x%x); "
-                                     "those records were kept", word);
-    if (word & 8u)
-        return fail(GEOCACHE_EINVAL, "a mesh face had a vertex index outside [0, n_verts) (status word 0x%x); "
-                                     "those faces were skipped", word);
-    if (word & 16u)
-        return fail(GEOCACHE_EINVAL, "a correspondence table index was outside [-1, H*W) (status word 0x%x); "
-                                     "those taps were dropped", word);
-    if (word) return fail(GEOCACHE_ETIMEOUT, "a bounded device wait gave up (status word 0x%x); outputs of that call are incomplete", word);
-    return ok();
-}
-
-const char* geocache_last_error(void) { return g_last_error.c_str(); }
-
-int geocache_debug_set_wait(uint64_t limit_ns, int drop_first_copy) {
-    geocache::set_debug_wait((unsigned long long)limit_ns, drop_first_copy);
-    return ok();
-}
-
-int geocache_build_corr(geocache_corr* c, void* stream) {
+// arguments of a build: sizes, required buffers, alignment and overlaps
+int check_build(const geocache_corr* c) {
     if (!c) return fail(GEOCACHE_EINVAL, "corr is NULL");
     int st = check_sizes(c->B, c->N, c->H, c->W);
     if (st) return st;
@@ -196,6 +152,69 @@ int geocache_build_corr(geocache_corr* c, void* stream) {
             if (overlap(c->src_ptr, ng, bufs[i], sizes[i]) || overlap(c->src_rec, nr, bufs[i], sizes[i]))
                 return fail(GEOCACHE_EALIAS, "the source index overlaps another buffer");
     }
+    return GEOCACHE_OK;
+}
+
+// the records of a corr whose keep masks and tile offsets are built, and its
+// source index when it has one
+int enqueue_records(const geocache_corr* c, cudaStream_t s) {
+    cudaError_t e = geocache::launch_fill_records(*c, s);
+    if (e != cudaSuccess) return cuda_fail(e, "record kernel launch");
+    if (c->src_ptr) {
+        e = geocache::launch_src_index(*c, s);
+        if (e != cudaSuccess) return cuda_fail(e, "source index kernel launch");
+    }
+    return ok();
+}
+
+}  // namespace
+
+int geocache::set_error(int status, const char* fmt, ...) {
+    char buf[512];
+    va_list ap;
+    va_start(ap, fmt);
+    vsnprintf(buf, sizeof buf, fmt, ap);
+    va_end(ap);
+    g_last_error = buf;
+    return status;
+}
+
+extern "C" {
+
+int geocache_abi_version(void) { return GEOCACHE_ABI_VERSION; }
+
+int geocache_device_status(void* stream) {
+    unsigned int word = 0, raster_word = 0;
+    cudaError_t e = geocache::read_device_error(&word, true, (cudaStream_t)stream);
+    if (e == cudaSuccess) e = geocache::read_raster_error(&raster_word, true, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "reading the device status word");
+    word |= raster_word;
+    if (word & 2u)
+        return fail(GEOCACHE_ESHAPE, "a sparse-form build had more records than max_records (status word 0x%x); "
+                                     "query geocache_corr_record_count and rebuild", word);
+    if (word & 4u)
+        return fail(GEOCACHE_EINVAL, "a record permutation entry was outside [0, max_records) (status word 0x%x); "
+                                     "those records were kept", word);
+    if (word & 8u)
+        return fail(GEOCACHE_EINVAL, "a mesh face had a vertex index outside [0, n_verts) (status word 0x%x); "
+                                     "those faces were skipped", word);
+    if (word & 16u)
+        return fail(GEOCACHE_EINVAL, "a correspondence table index was outside [-1, H*W) (status word 0x%x); "
+                                     "those taps were dropped", word);
+    if (word) return fail(GEOCACHE_ETIMEOUT, "a bounded device wait gave up (status word 0x%x); outputs of that call are incomplete", word);
+    return ok();
+}
+
+const char* geocache_last_error(void) { return g_last_error.c_str(); }
+
+int geocache_debug_set_wait(uint64_t limit_ns, int drop_first_copy) {
+    geocache::set_debug_wait((unsigned long long)limit_ns, drop_first_copy);
+    return ok();
+}
+
+int geocache_build_corr(geocache_corr* c, void* stream) {
+    const int st = check_build(c);
+    if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = geocache::launch_tau(c->pos, c->valid, c->B, c->N, c->H, c->W, c->tol_frac, c->tau, s);
     if (e != cudaSuccess) return cuda_fail(e, "tau kernel launch");
@@ -207,15 +226,15 @@ int geocache_build_corr(geocache_corr* c, void* stream) {
         e = geocache::launch_tile_ptr(*c, s);
         if (e != cudaSuccess) return cuda_fail(e, "tile-offset kernel launch");
     }
-    if (c->records) {
-        e = geocache::launch_fill_records(*c, s);
-        if (e != cudaSuccess) return cuda_fail(e, "record kernel launch");
-    }
-    if (c->src_ptr) {
-        e = geocache::launch_src_index(*c, s);
-        if (e != cudaSuccess) return cuda_fail(e, "source index kernel launch");
-    }
-    return ok();
+    return c->records ? enqueue_records(c, s) : ok();
+}
+
+int geocache_fill_records(geocache_corr* c, void* stream) {
+    const int st = check_build(c);
+    if (st) return st;
+    if (!c->keep || !c->tile_ptr || !c->records)
+        return fail(GEOCACHE_EINVAL, "filling records needs keep, tile_ptr and records");
+    return enqueue_records(c, (cudaStream_t)stream);
 }
 
 int geocache_corr_record_count(geocache_corr* c, int64_t* count, void* stream) {

@@ -72,7 +72,7 @@ EXPORTS = ("geocache_build_corr", "geocache_transport_step", "geocache_reconstru
            "geocache_transport_workspace", "geocache_transport_step_noalloc", "geocache_pack_anchors",
            "geocache_unpack_anchors", "geocache_transport_step_update", "geocache_permute_records",
            "geocache_raster_posmaps", "geocache_debug_set_wait", "geocache_raster_posmaps_supersampled",
-           "geocache_pool_posmaps",
+           "geocache_pool_posmaps", "geocache_fill_records",
            "geocache_last_error", "geocache_abi_version")
 
 
@@ -112,6 +112,8 @@ def load():
             getattr(L, name).restype = ctypes.c_int
         L.geocache_corr_record_count.argtypes = [ctypes.POINTER(Corr), ctypes.POINTER(ctypes.c_int64), P]
         L.geocache_corr_record_count.restype = ctypes.c_int
+        L.geocache_fill_records.argtypes = [ctypes.POINTER(Corr), P]
+        L.geocache_fill_records.restype = ctypes.c_int
         L.geocache_transport_workspace.argtypes = [ctypes.POINTER(Corr), i]
         L.geocache_transport_workspace.restype = ctypes.c_int64
         L.geocache_reconstruct.argtypes = [P, P, P, i, i64, ctypes.POINTER(Recon), P, P]
@@ -271,7 +273,11 @@ def build_sparse_corr(pos, valid, cams, K=4, tol_frac=0.01, tables=False, stream
         src_rec = torch.empty((records.shape[0], 2), dtype=torch.int32, device=dev)
     corr = make_corr(pos, valid, cams, tau, idx=idx, w=w, K=K, tol_frac=tol_frac, keep=keep, tile_ptr=tile_ptr,
                      records=records, mode=CORR_SPARSE, src_ptr=src_ptr, src_rec=src_rec)
-    return build_corr(corr, stream)
+    if tables:
+        return build_corr(corr, stream)
+    # the count left tau, the masks and the offsets: only the records are missing
+    _check(load().geocache_fill_records(ctypes.byref(corr.c), _stream(stream)))
+    return corr
 
 
 def make_recon(sampler="ddim", a_t=0.0, a_prev=0.0, sigma=0.0, sigma_next=0.0, pred_kind=None,
