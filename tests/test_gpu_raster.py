@@ -137,7 +137,7 @@ def test_bad_face_index_is_skipped_and_reported(gc):
     np.testing.assert_array_equal(pos.cpu().numpy()[0].view(np.uint32), ref_p.view(np.uint32))
 
 
-@pytest.mark.parametrize("s,H,W", [(2, 64, 64), (4, 32, 32), (8, 16, 16), (3, 24, 40)])
+@pytest.mark.parametrize("s,H,W", [(2, 64, 64), (4, 32, 32), (8, 16, 16), (3, 24, 40), (2, 21, 35), (4, 13, 27)])
 def test_supersampled_posmaps_bit_exact(gc, s, H, W):
     # rendered at s x the token grid and pooled to it (image-resolution maps
     # of Sec. 3.1 brought to the token grid of Sec. 3.2): validity and
@@ -183,6 +183,27 @@ def test_pool_posmaps_bit_exact(gc, s, H, W):
     np.testing.assert_array_equal(valid.cpu().numpy(), ref_v)
     np.testing.assert_array_equal(pos.cpu().numpy().view(np.uint32), ref_p.view(np.uint32))
     assert ref_v.mean() > 0.05
+
+
+@pytest.mark.parametrize("s,H,W", [(2, 19, 23), (4, 9, 31), (8, 5, 7), (5, 6, 11)])
+def test_pool_vector_rows_equal_scalar_ones(gc, s, H, W):
+    # random validity (whole rows and tokens of background among it), -0 and huge positions; the same maps 4 bytes
+    # (1 byte for the validity) off their alignment take the scalar path
+    rng = np.random.default_rng(s)
+    v = (rng.random((3, s * H, s * W)) < rng.choice([0.0, 0.3, 0.6, 1.0], (3, s * H, 1))).astype(np.uint8) * 5
+    x = rng.standard_normal(v.shape + (3,)).astype(np.float32)
+    x[rng.random(x.shape) < 0.05] = -0.0
+    x[0, 0, :3] = 3e38
+    x[v == 0] = np.nan
+    ref_p, ref_v = oracle.pool(x, v, s)
+    for off in (0, 1):
+        xs = torch.empty(x.size + 1, device="cuda")[off:off + x.size].view(x.shape)
+        vs = torch.empty(v.size + 1, dtype=torch.uint8, device="cuda")[off:off + v.size].view(v.shape)
+        xs.copy_(torch.from_numpy(x))
+        vs.copy_(torch.from_numpy(v))
+        pos, valid = gc.pool_posmaps(xs, vs, s)
+        np.testing.assert_array_equal(valid.cpu().numpy(), ref_v)
+        np.testing.assert_array_equal(pos.cpu().numpy().view(np.uint32), ref_p.view(np.uint32))
 
 
 def test_supersampled_posmaps_feed_the_correspondence_build(gc):
