@@ -1080,18 +1080,17 @@ cudaError_t launch_src_index(const geocache_corr& c, cudaStream_t s) {
 }
 
 // ------------------------------------------------- fused transport step --
-// One thread per quad of 4 consecutive tokens of one view (asset b, view v),
-// all channels in groups of 4.  For each group the thread issues 16-byte
-// loads of x0 (the anchor's fresh x0, or x0(t-1)) and of x_t first, then for
-// views outside the anchor set adds to each covered token the mean over the
-// covering anchors of the tap-weighted anchor increments (Eq. 1 with the
-// multi-anchor aggregation of Sec. 3.2; uncovered tokens keep x0(t-1)), then
-// stores x0(t) and the sampler reconstruction of every token.
-// Taps come from the keep masks (MODE = GEOCACHE_CORR_MASK: projection and
-// weights recomputed only for covered (token, anchor) pairs), from the full
-// per-tap tests (GEOMETRY) or from the tables (TABLE); all three are
-// bit-identical.  Streamed rows use evict-first hints so that the anchors'
-// rows, which the gathers re-read, stay in L2.
+// MASK, TABLE and GEOMETRY steps in one kernel each: a CTA streams the rows of
+// its tokens (x0: the anchor's fresh x0, or x0(t-1); x_t), for views outside the
+// anchor set adds to each covered token the mean over the covering anchors of
+// the tap-weighted anchor increments (Eq. 1 with the multi-anchor aggregation
+// of Sec. 3.2; uncovered tokens keep x0(t-1)), and stores x0(t) and the sampler
+// reconstruction of every token.
+// Taps come from the keep masks (MASK: projection and weights recomputed only
+// for covered (token, anchor) pairs), from the full per-tap tests (GEOMETRY) or
+// from the tables (TABLE); all three are bit-identical.  Rows that only stream
+// use evict-first hints so that the anchors' rows, which the gathers re-read,
+// stay in L2.
 constexpr int kThreads = 256;
 
 template <typename T>
@@ -1194,7 +1193,7 @@ __device__ __forceinline__ uint32_t quad_masks(const uint8_t* row, int cnt, bool
     return m;
 }
 
-// Fused cached step: a persistent kernel whose CTAs loop over work units
+// Large MASK steps: a persistent kernel whose CTAs loop over work units
 // (asset b, view v, tile of kTileTokens tokens, group of 4 channels).
 //  * Streaming: one thread arms the unit's mbarrier and issues TMA bulk
 //    copies (cp.async.bulk) of the unit's rows of x0 (the anchor's fresh x0,
@@ -1387,7 +1386,7 @@ __device__ __forceinline__ UnitCoord unit_coord(long long u, int n_tiles, int n_
 
 // Increments of the tile's covered tokens (views outside the anchor set),
 // left in sh.acc / sh.n for the tile's tokens.
-template <int K, int MODE, bool VEC>
+template <int K, bool VEC>
 __device__ __forceinline__ void tile_increments(const TransportArgs& args, FusedShared& sh, int b, int v, int tile0,
                                                 int cg, int cn) {
     const int HW = args.H * args.W;
@@ -1397,13 +1396,6 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     const int N = args.N, a = args.a;
     const size_t plane = (size_t)HW;
     const size_t tv0 = ((size_t)b * N + v) * plane;
-    float tau2 = 0.0f;
-    if (MODE == GEOCACHE_CORR_GEOMETRY) {
-        const float tu = __ldg(args.tau + b);
-        tau2 = __fmul_rn(tu, tu);
-    }
-    uint32_t fg = 0;
-    if (cnt > 0 && MODE == GEOCACHE_CORR_GEOMETRY) fg = quad_masks(args.valid + tv0 + p0, cnt, VEC);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         *reinterpret_cast<float4*>(sh.acc[4 * t + i]) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1411,30 +1403,21 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     }
     for (int ac = 0; ac < a; ac += kChunk) {
         const int na = a - ac < kChunk ? a - ac : kChunk;
-        if (MODE != GEOCACHE_CORR_TABLE)
-            for (int i = t; i < na * 16; i += kThreads)
-                reinterpret_cast<float*>(sh.cam)[i] = __ldg(
-                    reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (i >> 4)]) + (i & 15));
+        for (int i = t; i < na * 16; i += kThreads)
+            reinterpret_cast<float*>(sh.cam)[i] = __ldg(
+                reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (i >> 4)]) + (i & 15));
         // (token, anchor) work items of this anchor chunk
         uint32_t m4[4] = {0, 0, 0, 0};  // per own token: 4 bits per anchor of the chunk
         if (cnt > 0) {
-            if (MODE == GEOCACHE_CORR_MASK) {
-                const uint8_t* krow = args.keep + ((size_t)b * N + v) * N * plane + p0;
-                uint32_t q[kChunk];
+            const uint8_t* krow = args.keep + ((size_t)b * N + v) * N * plane + p0;
+            uint32_t q[kChunk];
 #pragma unroll
-                for (int s2 = 0; s2 < kChunk; ++s2)  // the chunk's masks in flight together
-                    q[s2] = s2 < na ? quad_masks(krow + (size_t)args.anchors[ac + s2] * plane, cnt, VEC) : 0u;
+            for (int s2 = 0; s2 < kChunk; ++s2)  // the chunk's masks in flight together
+                q[s2] = s2 < na ? quad_masks(krow + (size_t)args.anchors[ac + s2] * plane, cnt, VEC) : 0u;
 #pragma unroll
-                for (int s2 = 0; s2 < kChunk; ++s2)
+            for (int s2 = 0; s2 < kChunk; ++s2)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) m4[i] |= ((q[s2] >> (8 * i)) & 15u) << (4 * s2);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const bool cand = MODE == GEOCACHE_CORR_GEOMETRY ? ((fg >> (8 * i)) & 0xffu) != 0 : i < cnt;
-                    if (cand) m4[i] = (1u << (4 * na)) - 1u;  // every anchor is a candidate
-                }
-            }
+                for (int i = 0; i < 4; ++i) m4[i] |= ((q[s2] >> (8 * i)) & 15u) << (4 * s2);
         }
         int mine = 0;
 #pragma unroll
@@ -1461,7 +1444,7 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
                 const int s_loc = (int)((it >> 10) & 63u);
                 const int m = (int)((it >> 16) & 15u);
                 Taps tp;
-                item_taps<K, MODE>(args, sh.cam[s_loc], b, v, ac + s_loc, tile0 + lp, m, tv0, plane, tau2, tp);
+                item_taps<K, GEOCACHE_CORR_MASK>(args, sh.cam[s_loc], b, v, ac + s_loc, tile0 + lp, m, tv0, plane, 0.0f, tp);
                 if (tp.kept) {
                     item_increment<K>(args, tp, b, ac + s_loc, cg, cn, plane, g);
                     s_mine = s_loc;
@@ -1485,7 +1468,7 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     }
 }
 
-template <typename T, int K, int MODE>
+template <typename T, int K>
 __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const TransportArgs args, int n_tiles, int n_cg,
                                                                    long long n_units) {
     __shared__ FusedShared sh;
@@ -1541,7 +1524,7 @@ __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const Transpo
         const int cnt = p0 < HW ? (HW - p0 < 4 ? HW - p0 : 4) : 0;
         const int cn = C - c.cg < 4 ? C - c.cg : 4;
         const int slot = args.slot_of[c.v];
-        if (slot < 0) tile_increments<K, MODE, true>(args, sh, c.b, c.v, tile0, c.cg, cn);
+        if (slot < 0) tile_increments<K, true>(args, sh, c.b, c.v, tile0, c.cg, cn);
 
         const bool ok = mbar_wait_bounded(&sh.bar[st], parity[st], args.wait_limit_ns);
         if (__syncthreads_or(!ok)) {  // the whole CTA gives up together
@@ -1605,7 +1588,7 @@ __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const Transpo
 // General path (sizes the bulk copies cannot serve: H*W not a multiple of 8
 // or buffers not 16-byte aligned): one CTA per unit, registers instead of
 // the shared-memory ring.
-template <typename T, int K, int MODE, bool VEC>
+template <typename T, int K, bool VEC>
 __global__ void __launch_bounds__(kThreads) transport_simple_kernel(const TransportArgs args, int n_tiles, int n_cg) {
     __shared__ FusedShared sh;
     const int t = threadIdx.x;
@@ -1637,7 +1620,7 @@ __global__ void __launch_bounds__(kThreads) transport_simple_kernel(const Transp
             if (recon) xt[cc] = Lat4<T>::load_raw(xt_p, view_base + (size_t)(c.cg + cc) * plane, cnt, VEC);
         }
     }
-    if (slot < 0) tile_increments<K, MODE, VEC>(args, sh, c.b, c.v, tile0, c.cg, cn);
+    if (slot < 0) tile_increments<K, VEC>(args, sh, c.b, c.v, tile0, c.cg, cn);
     if (cnt <= 0) return;
     if (slot < 0) {
 #pragma unroll
@@ -1669,6 +1652,162 @@ __global__ void __launch_bounds__(kThreads) transport_simple_kernel(const Transp
             const size_t e = view_base + (size_t)(c.cg + cc) * plane;
             Lat4<T>::store(xn_p, e, cnt, VEC, y);
             if (args.pred_out) Lat4<float>::store(args.pred_out, e, cnt, VEC, pr);
+        }
+    }
+}
+
+// Quotient by a divisor fixed for a launch, as a multiply-high and a shift
+// (Granlund and Montgomery, division by invariant integers using
+// multiplication): with l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1,
+// n / d = (umulhi(m, n) + n) >> l for 0 <= n < 2^31.  The CTAs of a launch
+// split their block index into (asset, view, tile, channel group, ...) with
+// these instead of integer divisions.
+struct FastDiv {
+    uint32_t d, m, l;
+    __device__ __forceinline__ uint32_t quo(uint32_t n) const { return (__umulhi(m, n) + n) >> l; }
+};
+static FastDiv make_fastdiv(uint32_t d) {
+    FastDiv f{d, 0u, 0u};
+    while ((1ull << f.l) < d) ++f.l;
+    f.m = (uint32_t)(((1ull << 32) * ((1ull << f.l) - d)) / d + 1);
+    return f;
+}
+
+// TABLE and GEOMETRY steps, and MASK steps of few units: one CTA per 256 tokens
+// of a view and group of 4 channels, one token per thread, any alignment.
+// The two kernels above take a tile of 1024 tokens per CTA, whose work items
+// (token, anchor; up to 4 per token and round of anchors) go 256 at a time
+// through a chain of dependent loads with a barrier per anchor; where their
+// units do not fill the GPU several times over, the chains of a covered tile
+// are the time of the call.  Here the items of a CTA are a quarter as many, and
+// each writes its increment to the slot of its (anchor, token), so that no
+// barrier orders them: every thread then sums its token's slots in anchor
+// order (the same additions).  8 assets x 6 views of 96 x 96 x 4 bf16, 3 anchors,
+// against those kernels: masks 19.7 -> 12.0 us, tables (every token an item)
+// 50.4 -> 19.1, geometry 48.8 -> 17.9; 64 assets: tables 215 -> 144, geometry
+// 199 -> 137, so those take it at every size.
+constexpr int kTokenAnchors = 4;  // anchors per round
+// resident CTAs per SM: 3 (80 registers, a few spilled) or 2, whichever was
+// faster: 8 assets, masks 12.0 / 12.2, geometry 17.9 / 17.9 (64 assets 137 / 155),
+// tables 20.4 / 19.1, f32 masks 9.2 / 8.1 (4 assets); 4 were slower
+template <typename T, int MODE>
+constexpr int kTokenBlocks = MODE == GEOCACHE_CORR_TABLE || (MODE == GEOCACHE_CORR_MASK && sizeof(T) == 4) ? 2 : 3;
+
+template <typename T, int K, int MODE>
+__global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_token_kernel(const TransportArgs args, FastDiv n_cg) {
+    __shared__ float4 s_g[kTokenAnchors][kThreads];     // increments of the round's (anchor, token)s
+    __shared__ uint8_t s_has[kTokenAnchors][kThreads];  // whether the anchor covers the token
+    __shared__ uint32_t s_item[kTokenAnchors * kThreads];  // token | anchor << 10 | keep mask << 16
+    __shared__ geocache_camera s_cam[kTokenAnchors];
+    __shared__ int s_wcnt[kThreads / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int HW = args.H * args.W, N = args.N, C = args.C, a = args.a;
+    const size_t plane = (size_t)HW;
+    const int tile = (int)n_cg.quo(blockIdx.x), cg = ((int)blockIdx.x - tile * (int)n_cg.d) * 4;
+    const int v = blockIdx.y, b = blockIdx.z;
+    const int p0 = tile * kThreads, p = p0 + t;
+    const bool in = p < HW;
+    const int cn = C - cg < 4 ? C - cg : 4;
+    const int slot = args.slot_of[v];
+    const bool recon = args.coef.enabled;
+    const size_t base = (((size_t)b * N + v) * C + cg) * plane + p;
+    const float* src = slot >= 0 ? args.x0_new + (((size_t)b * a + slot) * C + cg) * plane + p : args.x0_prev + base;
+    const T* xt_p = static_cast<const T*>(args.x_t);
+    float x0[4], xt[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        x0[c] = in && c < cn ? __ldg(src + (size_t)c * plane) : 0.0f;
+        xt[c] = in && c < cn && recon ? lat_load(xt_p, base + (size_t)c * plane) : 0.0f;
+    }
+    if (slot < 0) {
+        const size_t tv0 = ((size_t)b * N + v) * plane;
+        float tau2 = 0.0f;
+        if (MODE == GEOCACHE_CORR_GEOMETRY) {
+            const float tu = __ldg(args.tau + b);
+            tau2 = __fmul_rn(tu, tu);
+        }
+        const bool fg = in && (MODE != GEOCACHE_CORR_GEOMETRY || __ldg(args.valid + tv0 + p) != 0);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        int n = 0;
+        for (int ac = 0; ac < a; ac += kTokenAnchors) {
+            const int na = a - ac < kTokenAnchors ? a - ac : kTokenAnchors;
+            if (MODE != GEOCACHE_CORR_TABLE && t < na * 16)
+                reinterpret_cast<float*>(s_cam)[t] = __ldg(
+                    reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (t >> 4)]) + (t & 15));
+            // the round's candidate (anchor, token)s, listed by warp
+            uint32_t m[kTokenAnchors], kept[kTokenAnchors];
+            int mine = 0;
+#pragma unroll
+            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                m[s2] = 0;
+                if (s2 < na && fg)
+                    m[s2] = MODE == GEOCACHE_CORR_MASK
+                                ? __ldg(args.keep + (((size_t)b * N + v) * N + args.anchors[ac + s2]) * plane + p)
+                                : 15u;
+            }
+#pragma unroll
+            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                kept[s2] = __ballot_sync(0xffffffffu, m[s2] & 15u);
+                mine += __popc(kept[s2]);
+                s_has[s2][t] = 0;
+            }
+            if (lane == 0) s_wcnt[warp] = mine;
+            __syncthreads();
+            int at = 0, n_items = 0;
+#pragma unroll
+            for (int w = 0; w < kThreads / 32; ++w) {
+                at += w < warp ? s_wcnt[w] : 0;
+                n_items += s_wcnt[w];
+            }
+#pragma unroll
+            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                if (m[s2] & 15u)
+                    s_item[at + __popc(kept[s2] & ((1u << lane) - 1u))] =
+                        (uint32_t)t | ((uint32_t)s2 << 10) | ((m[s2] & 15u) << 16);
+                at += __popc(kept[s2]);
+            }
+            __syncthreads();
+            for (int j = t; j < n_items; j += kThreads) {
+                const uint32_t it = s_item[j];
+                const int lp = (int)(it & 1023u), s2 = (int)((it >> 10) & 63u);
+                Taps tp;
+                item_taps<K, MODE>(args, s_cam[s2], b, v, ac + s2, p0 + lp, (int)(it >> 16), tv0, plane, tau2, tp);
+                if (tp.kept) {
+                    float g[4];
+                    item_increment<K>(args, tp, b, ac + s2, cg, cn, plane, g);
+                    s_g[s2][lp] = make_float4(g[0], g[1], g[2], g[3]);
+                    s_has[s2][lp] = 1;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                if (!s_has[s2][t]) continue;
+                const float4 g = s_g[s2][t];
+                acc[0] = __fadd_rn(acc[0], g.x);
+                acc[1] = __fadd_rn(acc[1], g.y);
+                acc[2] = __fadd_rn(acc[2], g.z);
+                acc[3] = __fadd_rn(acc[3], g.w);
+                ++n;
+            }
+            // the next round clears a thread's own flags and writes the slots two barriers later
+        }
+        if (n) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) x0[c] = fold_one(args.update == GEOCACHE_UPDATE_COPY, x0[c], acc[c], n);
+        }
+    }
+    if (!in) return;
+    T* xn_p = static_cast<T*>(args.x_next);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (c >= cn) break;
+        const size_t e = base + (size_t)c * plane;
+        if (slot < 0 || args.write_anchor_rows) args.x0_out[e] = x0[c];
+        if (recon) {
+            float pr;
+            lat_store(xn_p, e, recon_one(args.coef, xt[c], x0[c], pr));
+            if (args.pred_out) args.pred_out[e] = pr;
         }
     }
 }
@@ -1776,23 +1915,6 @@ struct QuadRows {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-
-// Quotient by a divisor fixed for a launch, as a multiply-high and a shift
-// (Granlund and Montgomery, division by invariant integers using
-// multiplication): with l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1,
-// n / d = (umulhi(m, n) + n) >> l for 0 <= n < 2^31.  The CTAs of a launch
-// split their block index into (asset, view, tile, channel group, ...) with
-// these instead of integer divisions.
-struct FastDiv {
-    uint32_t d, m, l;
-    __device__ __forceinline__ uint32_t quo(uint32_t n) const { return (__umulhi(m, n) + n) >> l; }
-};
-static FastDiv make_fastdiv(uint32_t d) {
-    FastDiv f{d, 0u, 0u};
-    while ((1ull << f.l) < d) ++f.l;
-    f.m = (uint32_t)(((1ull << 32) * ((1ull << f.l) - d)) / d + 1);
-    return f;
-}
 
 // Grid shape of a sparse step's launches and the divisors that split it.
 struct SparseGrid {
@@ -2389,8 +2511,23 @@ static int persistent_grid(Kern kern, size_t dyn_smem) {
     return sms * (per_sm > 0 ? per_sm : 1);
 }
 
+// Units (tiles of 1024 tokens x channel groups) up to which a MASK step takes
+// one token per thread: with 16-byte aligned rows, against the staged kernel
+// (us; 3 anchors, 96 x 96 x 4 bf16): 24 units 9.0 -> 4.4, 432 19.7 -> 12.0, 864
+// 30.7 -> 28.0, but 1,728 49.1 -> 53.9; otherwise against one CTA per tile
+// (75 x 53 x 4): 96 units 8.2 -> 5.1, 384 11.9 -> 11.1, but 960 23.7 -> 29.2.
+constexpr long long kTokenUnitsStaged = 1024, kTokenUnitsSimple = 384;
+
 template <typename T, int K, int MODE>
-static cudaError_t launch_quad(const TransportArgs& t, cudaStream_t s) {
+static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s) {
+    const int HW = t.H * t.W, n_cg = (t.C + 3) / 4;
+    const dim3 grid((unsigned)((HW + kThreads - 1) / kThreads * n_cg), t.N, t.B);
+    transport_token_kernel<T, K, MODE><<<grid, kThreads, 0, s>>>(t, make_fastdiv((uint32_t)n_cg));
+    return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t launch_mask(const TransportArgs& t, cudaStream_t s) {
     const int HW = t.H * t.W;
     const uintptr_t al = (uintptr_t)t.x0_new | (uintptr_t)t.x0_prev | (uintptr_t)t.x0_out | (uintptr_t)t.x_t |
                          (uintptr_t)t.x_next | (uintptr_t)t.pred_out | (uintptr_t)t.keep | (uintptr_t)t.valid;
@@ -2398,13 +2535,17 @@ static cudaError_t launch_quad(const TransportArgs& t, cudaStream_t s) {
     const int n_tiles = (HW + kTileTokens - 1) / kTileTokens;
     const int n_cg = (t.C + 3) / 4;
     const long long n_units = (long long)t.B * t.N * n_tiles * n_cg;
+    const bool staged = vec && HW % 8 == 0;
+    // (a pending request of the test hook is for the staged kernel)
+    if (n_units <= (staged ? kTokenUnitsStaged : kTokenUnitsSimple) && !(staged && g_drop_first_copy.load()))
+        return launch_token<T, K, GEOCACHE_CORR_MASK>(t, s);
     // TMA bulk rows need 16-byte aligned starts and sizes: HW % 8 == 0 covers bf16 rows
-    if (vec && HW % 8 == 0) {
+    if (staged) {
         TransportArgs ta = t;
         ta.wait_limit_ns = g_wait_limit_ns.load();
         ta.drop_first_copy = g_drop_first_copy.exchange(0);
         const size_t dyn = kStages * 4 * kTileTokens * (sizeof(float) + sizeof(T));
-        auto kern = transport_fused_kernel<T, K, MODE>;
+        auto kern = transport_fused_kernel<T, K>;
         static int grid = 0;  // per instantiation and process (one device per process)
         if (!grid) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -2418,9 +2559,9 @@ static cudaError_t launch_quad(const TransportArgs& t, cudaStream_t s) {
     }
     if (n_units > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (vec)
-        transport_simple_kernel<T, K, MODE, true><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
+        transport_simple_kernel<T, K, true><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
     else
-        transport_simple_kernel<T, K, MODE, false><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
+        transport_simple_kernel<T, K, false><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
     return cudaGetLastError();
 }
 
@@ -2428,9 +2569,9 @@ template <typename T, int K>
 static cudaError_t launch_transport_t(const TransportArgs& t, cudaStream_t s) {
     switch (t.mode) {
         case GEOCACHE_CORR_SPARSE: return launch_sparse<T, K>(t, s);
-        case GEOCACHE_CORR_MASK: return launch_quad<T, K, GEOCACHE_CORR_MASK>(t, s);
-        case GEOCACHE_CORR_TABLE: return launch_quad<T, K, GEOCACHE_CORR_TABLE>(t, s);
-        default: return launch_quad<T, K, GEOCACHE_CORR_GEOMETRY>(t, s);
+        case GEOCACHE_CORR_MASK: return launch_mask<T, K>(t, s);
+        case GEOCACHE_CORR_TABLE: return launch_token<T, K, GEOCACHE_CORR_TABLE>(t, s);
+        default: return launch_token<T, K, GEOCACHE_CORR_GEOMETRY>(t, s);
     }
 }
 

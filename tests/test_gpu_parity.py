@@ -210,6 +210,44 @@ def test_corr_modes_agree_bitwise(gc, workloads, name, K):
     np.testing.assert_array_equal(got_mask, got_tab)
 
 
+@pytest.mark.parametrize("B,N,H,W,C,a,K,dtype,update,in_place", [
+    (1, 6, 16, 16, 4, 2, 4, "bf16", "delta", False),    # one tile of 256 tokens, exactly
+    (2, 6, 37, 29, 5, 5, 4, "bf16", "delta", True),     # ragged, two rounds of anchors, a channel group of 1
+    (3, 12, 24, 40, 3, 9, 1, "f32", "copy", False),     # three rounds
+    (86, 6, 36, 32, 4, 2, 4, "bf16", "delta", False),   # 1,032 units with a last tile of 128 tokens: staged
+    (85, 6, 36, 32, 4, 3, 4, "f32", "copy", True),      # 1,020 units: one token per thread
+    (33, 6, 37, 29, 4, 3, 4, "bf16", "copy", True),     # 396 units, unaligned rows: one CTA per tile
+    (32, 6, 37, 29, 4, 2, 1, "f32", "delta", False),    # 384 units
+])
+def test_mode_kernels_agree_bitwise(gc, B, N, H, W, C, a, K, dtype, update, in_place):
+    # every kernel that the MASK, TABLE and GEOMETRY steps choose between, against the sparse step
+    base = dict(B=3, H=H, W=W, N=N, layout="hunyuan6" if N == 6 else "ring8_polar4")
+    w = synth.replicate_assets(synth.make_workload("batch128", **base), B)
+    pos, valid, cams = (torch.from_numpy(x).cuda() for x in (w.pos, w.valid, w.cams))
+    sparse = gc.build_sparse_corr(pos, valid, cams, K=K, tables=True)
+    gen = torch.Generator("cuda").manual_seed(3)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    anchors = sorted(np.random.default_rng(a).choice(N, a, replace=False).tolist())
+    x0, x_t = rnd(B, N, C, H, W), rnd(B, N, C, H, W).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    x0_new = (x0[:, anchors] + 0.1 * rnd(B, a, C, H, W)).contiguous()
+    outs = {}
+    for mode in (gc.CORR_SPARSE, gc.CORR_MASK, gc.CORR_TABLE, gc.CORR_GEOMETRY):
+        c = gc.make_corr(pos, valid, cams, sparse.tau, sparse.idx, sparse.w, K=K, mode=mode, keep=sparse.keep,
+                         tile_ptr=sparse._keep["tile_ptr"], records=sparse._keep["records"])
+        prev, xt = x0.clone(), x_t.clone()
+        out, xn = (prev, xt) if in_place else (torch.empty_like(prev), torch.empty_like(xt))
+        pred = torch.empty_like(x0)
+        r = gc.make_recon("fm_euler", sigma=0.6, sigma_next=0.5, pred_kind="velocity", pred_out=pred)
+        ws = torch.empty(max(4, c.workspace_floats(C)), device="cuda") if mode == gc.CORR_SPARSE else None
+        gc.transport_step(c, anchors, C, x0_new, prev, out, xt, xn, r, workspace=ws, update=update)
+        outs[mode] = [x.clone() for x in (out, xn, pred)]
+    gc.device_status()
+    assert (outs[gc.CORR_SPARSE][0] != x0).any()
+    for mode in (gc.CORR_MASK, gc.CORR_TABLE, gc.CORR_GEOMETRY):
+        for x, y in zip(outs[mode], outs[gc.CORR_SPARSE]):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+
 @pytest.mark.parametrize("pred", ["eps", "v"])
 def test_ddim_prediction_outputs(gc, workloads, pred):
     w = workloads("hunyuan64")
