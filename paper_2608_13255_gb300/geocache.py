@@ -10,6 +10,7 @@ been built, every call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -144,6 +145,9 @@ def _check(status: int):
 
 def _stream(stream):
     if stream is None:
+        # the current stream's handle without a Stream object around it (3.1 -> 0.3 us a call)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, torch.cuda.Stream):
         return ctypes.c_void_p(stream.cuda_stream)
@@ -153,6 +157,9 @@ def _stream(stream):
 def _dev(t, dtype, numel=None, name="tensor"):
     if t is None:
         return None
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (
+            numel is None or t.numel() == numel):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor):
         raise TypeError("%s must be a torch tensor" % name)
     if not t.is_cuda:
@@ -161,9 +168,7 @@ def _dev(t, dtype, numel=None, name="tensor"):
         raise TypeError("%s must be %s (got %s)" % (name, dtype, t.dtype))
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
-    if numel is not None and t.numel() != numel:
-        raise ValueError("%s has %d elements, expected %d" % (name, t.numel(), numel))
-    return t.data_ptr()
+    raise ValueError("%s has %d elements, expected %d" % (name, t.numel(), numel))
 
 
 def _lat_dtype(t):
@@ -256,27 +261,27 @@ def build_sparse_corr(pos, valid, cams, K=4, tol_frac=0.01, tables=False, stream
     never per step."""
     B, N, H, W = valid.shape
     dev = pos.device
-    tau = torch.zeros(B, dtype=torch.float32, device=dev)
+    tau = torch.empty(B, dtype=torch.float32, device=dev)
     keep = torch.empty((B, N, N, H, W), dtype=torch.uint8, device=dev)
     tile_ptr = torch.empty(B * N * N * tiles_per_view(H, W) + 1, dtype=torch.int32, device=dev)
-    c0 = make_corr(pos, valid, cams, tau, K=K, tol_frac=tol_frac, keep=keep, tile_ptr=tile_ptr,
-                   mode=CORR_MASK)
-    R = record_count(c0, stream)
+    corr = make_corr(pos, valid, cams, tau, K=K, tol_frac=tol_frac, keep=keep, tile_ptr=tile_ptr, mode=CORR_MASK)
+    R = record_count(corr, stream)
     records = torch.empty((max(R, 1), 4), dtype=torch.int32, device=dev)
-    idx = w = None
+    c, refs = corr.c, corr._keep
+    refs["records"], c.records, c.max_records = records, records.data_ptr(), records.shape[0]
+    c.mode = CORR_SPARSE
     if tables:
-        idx = torch.empty((B, N, N, H, W, K), dtype=torch.int32, device=dev)
-        w = torch.empty((B, N, N, H, W, K), dtype=torch.float32, device=dev)
-    src_ptr = src_rec = None
+        refs["idx"] = torch.empty((B, N, N, H, W, K), dtype=torch.int32, device=dev)
+        refs["w"] = torch.empty((B, N, N, H, W, K), dtype=torch.float32, device=dev)
+        c.idx, c.w = refs["idx"].data_ptr(), refs["w"].data_ptr()
     if source_index:
-        src_ptr = torch.empty(B * N * tiles_per_view(H, W) + 1, dtype=torch.int32, device=dev)
-        src_rec = torch.empty((records.shape[0], 2), dtype=torch.int32, device=dev)
-    corr = make_corr(pos, valid, cams, tau, idx=idx, w=w, K=K, tol_frac=tol_frac, keep=keep, tile_ptr=tile_ptr,
-                     records=records, mode=CORR_SPARSE, src_ptr=src_ptr, src_rec=src_rec)
+        refs["src_ptr"] = torch.empty(B * N * tiles_per_view(H, W) + 1, dtype=torch.int32, device=dev)
+        refs["src_rec"] = torch.empty((records.shape[0], 2), dtype=torch.int32, device=dev)
+        c.src_ptr, c.src_rec = refs["src_ptr"].data_ptr(), refs["src_rec"].data_ptr()
     if tables:
         return build_corr(corr, stream)
     # the count left tau, the masks and the offsets: only the records are missing
-    _check(load().geocache_fill_records(ctypes.byref(corr.c), _stream(stream)))
+    _check(load().geocache_fill_records(ctypes.byref(c), _stream(stream)))
     return corr
 
 
@@ -298,13 +303,23 @@ _SCHED_KINDS = {"every_k": SCHED_EVERY_K, "head_mid_tail": SCHED_HEAD_MID_TAIL, 
                 "all_full": SCHED_ALL_FULL, "single_cached": SCHED_SINGLE_CACHED}
 
 
+def _schedule_values(spec: dict):
+    get = spec.get
+    return (_SCHED_KINDS[spec["kind"]], int(get("k", 1)), int(get("head", 2)), int(get("mid", 1)),
+            int(get("tail", 1)), tuple(get("steps", ())), int(get("contiguous", 0)))
+
+
+def _make_schedule(kind, k, head, mid, tail, steps, contiguous):
+    arr = (ctypes.c_int32 * max(1, len(steps)))(*steps)
+    return Schedule(kind, k, head, mid, tail, ctypes.cast(arr, ctypes.c_void_p), len(steps), contiguous), arr
+
+
+# the C structs of the schedules last asked about, by their values; the calls only read them
+_schedule = functools.lru_cache(maxsize=64)(_make_schedule)
+
+
 def make_schedule(spec: dict):
-    kind = _SCHED_KINDS[spec["kind"]]
-    steps = (ctypes.c_int32 * max(1, len(spec.get("steps", ()))))(*spec.get("steps", ()))
-    s = Schedule(kind, int(spec.get("k", 1)), int(spec.get("head", 2)), int(spec.get("mid", 1)),
-                 int(spec.get("tail", 1)), ctypes.cast(steps, ctypes.c_void_p), len(spec.get("steps", ())),
-                 int(spec.get("contiguous", 0)))
-    return s, steps
+    return _make_schedule(*_schedule_values(spec))
 
 
 # ---------------------------------------------------------- entry points --
@@ -323,25 +338,25 @@ def transport_step(corr: CorrHandle, anchors, C, x0_anchor_new, x0_prev, x0_out,
     geocache_transport_step_update (update="copy", the value-copy ablation)
     on torch tensors (see include/geocache.h)."""
     c = corr.c
-    anc = sorted(int(a) for a in anchors)
+    anc = sorted(map(int, anchors))
     a = len(anc)
-    n_all = c.B * c.N * C * c.H * c.W
+    C = int(C)
+    per = C * c.H * c.W
+    n_anc, n_all = c.B * a * per, c.B * c.N * per
     arr = (ctypes.c_int32 * max(1, a))(*anc)
     lat = F32
-    pt = pn = None
+    pt = pn = r = None
     if recon is not None:
         lat = _lat_dtype(x_t)
         dt = x_t.dtype
         pt, pn = _dev(x_t, dt, n_all, "x_t"), _dev(x_next, dt, n_all, "x_next")
         _check_pred(recon, n_all)
-    st = load().geocache_transport_step_update(
-        ctypes.byref(c), UPDATES[update], ctypes.cast(arr, ctypes.c_void_p), a, int(C),
-        _dev(x0_anchor_new, torch.float32, c.B * a * C * c.H * c.W, "x0_anchor_new"),
-        _dev(x0_prev, torch.float32, n_all, "x0_prev"), _dev(x0_out, torch.float32, n_all, "x0_out"),
-        pt, pn, lat, ctypes.byref(recon) if recon is not None else None,
-        _dev(workspace, torch.float32, None, "workspace"), 0 if workspace is None else workspace.numel(),
-        _stream(stream))
-    _check(st)
+        r = ctypes.byref(recon)
+    f32 = torch.float32
+    _check(load().geocache_transport_step_update(
+        ctypes.byref(c), UPDATES[update], arr, a, C, _dev(x0_anchor_new, f32, n_anc, "x0_anchor_new"),
+        _dev(x0_prev, f32, n_all, "x0_prev"), _dev(x0_out, f32, n_all, "x0_out"), pt, pn, lat, r,
+        _dev(workspace, f32, None, "workspace"), 0 if workspace is None else workspace.numel(), _stream(stream)))
 
 
 def permute_records(corr: CorrHandle, perm, out=None, stream=None) -> CorrHandle:
@@ -447,30 +462,30 @@ def transport_step_noalloc(corr: CorrHandle, anchors, C, x0_anchor_new, x0_prev,
 def _rows(src_full, a):
     if src_full.dim() < 2:
         raise ValueError("per-view tensors are [B, N, ...]")
-    B, N = src_full.shape[0], src_full.shape[1]
-    return B, N, (src_full[0, 0].numel() if B * N else 0) * src_full.element_size()
+    B, N = src_full.shape[:2]
+    return B, N, (src_full.numel() // (B * N) if B * N else 0) * src_full.element_size()
 
 
 def pack_anchors(src, dst, anchors, stream=None):
     """geocache_pack_anchors: dst [B, a, ...] <- src[:, anchors] (raw bytes)."""
     anc = sorted(int(x) for x in anchors)
     B, N, row = _rows(src, len(anc))
-    if dst.dtype != src.dtype or tuple(dst.shape) != (B, len(anc)) + tuple(src.shape[2:]):
+    if dst.dtype != src.dtype or dst.shape != (B, len(anc)) + src.shape[2:]:
         raise ValueError("dst must be [B, a, ...] of src's dtype")
     arr = (ctypes.c_int32 * len(anc))(*anc)
     _check(load().geocache_pack_anchors(_dev(src, src.dtype, name="src"), _dev(dst, dst.dtype, name="dst"), row, B, N,
-                                        ctypes.cast(arr, ctypes.c_void_p), len(anc), _stream(stream)))
+                                        arr, len(anc), _stream(stream)))
 
 
 def unpack_anchors(src, dst, anchors, stream=None):
     """geocache_unpack_anchors: dst[:, anchors] <- src [B, a, ...] (raw bytes)."""
     anc = sorted(int(x) for x in anchors)
     B, N, row = _rows(dst, len(anc))
-    if src.dtype != dst.dtype or tuple(src.shape) != (B, len(anc)) + tuple(dst.shape[2:]):
+    if src.dtype != dst.dtype or src.shape != (B, len(anc)) + dst.shape[2:]:
         raise ValueError("src must be [B, a, ...] of dst's dtype")
     arr = (ctypes.c_int32 * len(anc))(*anc)
     _check(load().geocache_unpack_anchors(_dev(src, src.dtype, name="src"), _dev(dst, dst.dtype, name="dst"), row, B, N,
-                                          ctypes.cast(arr, ctypes.c_void_p), len(anc), _stream(stream)))
+                                          arr, len(anc), _stream(stream)))
 
 
 def reconstruct(x_t, x0, x_next, recon: Recon, x0_store=None, stream=None):
@@ -484,7 +499,7 @@ def reconstruct(x_t, x0, x_next, recon: Recon, x0_store=None, stream=None):
 
 
 def is_full_step(step: int, S: int, sched: dict) -> bool:
-    s, _keep = make_schedule(sched)
+    s, _keep = _schedule(*_schedule_values(sched))
     r = load().geocache_is_full_step(int(step), int(S), ctypes.byref(s))
     if r < 0:
         raise GeocacheError(r, last_error())
@@ -493,11 +508,11 @@ def is_full_step(step: int, S: int, sched: dict) -> bool:
 
 def rotate_anchors(N: int, a: int, step: int, S: int, sched: dict):
     """(anchors, is_full) of a step."""
-    s, _keep = make_schedule(sched)
+    s, _keep = _schedule(*_schedule_values(sched))
     out = (ctypes.c_int32 * a)()
     full = ctypes.c_int(0)
-    _check(load().geocache_rotate_anchors(int(N), int(a), int(step), int(S), ctypes.byref(s),
-                                          ctypes.cast(out, ctypes.c_void_p), ctypes.byref(full)))
+    _check(load().geocache_rotate_anchors(int(N), int(a), int(step), int(S), ctypes.byref(s), out,
+                                          ctypes.byref(full)))
     return list(out), bool(full.value)
 
 
