@@ -1673,7 +1673,16 @@ static FastDiv make_fastdiv(uint32_t d) {
     return f;
 }
 
-// TABLE and GEOMETRY steps, and MASK steps of few units: one CTA per 256 tokens
+// Tile offset i of the sparse form clamped to the records that exist, [0,
+// cap]: a build whose records overflowed the capacity or the int32 offsets
+// is flagged in the status word, and the transport then reads only records
+// that exist.
+__device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_ptr, size_t i, long long cap) {
+    const long long x = __ldg(tile_ptr + i);
+    return (int)(x < 0 ? 0 : (x < cap ? x : cap));
+}
+
+// TABLE and GEOMETRY steps, and MASK and SPARSE steps of few units: one CTA per 256 tokens
 // of a view and group of 4 channels, one token per thread, any alignment.
 // The two kernels above take a tile of 1024 tokens per CTA, whose work items
 // (token, anchor; up to 4 per token and round of anchors) go 256 at a time
@@ -1700,6 +1709,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
     __shared__ uint32_t s_item[kTokenAnchors * kThreads];  // token | anchor << 10 | keep mask << 16
     __shared__ geocache_camera s_cam[kTokenAnchors];
     __shared__ int s_wcnt[kThreads / 32];
+    __shared__ int s_r0[kTokenAnchors], s_rn[kTokenAnchors];  // SPARSE: the tile's records of the round's anchors
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int HW = args.H * args.W, N = args.N, C = args.C, a = args.a;
     const size_t plane = (size_t)HW;
@@ -1731,55 +1741,92 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
         int n = 0;
         for (int ac = 0; ac < a; ac += kTokenAnchors) {
             const int na = a - ac < kTokenAnchors ? a - ac : kTokenAnchors;
-            if (MODE != GEOCACHE_CORR_TABLE && t < na * 16)
-                reinterpret_cast<float*>(s_cam)[t] = __ldg(
-                    reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (t >> 4)]) + (t & 15));
-            // the round's candidate (anchor, token)s, listed by warp
-            uint32_t m[kTokenAnchors], kept[kTokenAnchors];
-            int mine = 0;
+            if (MODE == GEOCACHE_CORR_SPARSE) {
+                // the records of the 1024-token tile around the CTA's tokens; they are in token order, so a
+                // warp's are mostly all its CTA's or all another's
+                if (t < kTokenAnchors) {
+                    int r0 = 0, r1 = 0;
+                    if (t < na) {
+                        const size_t i = (((size_t)b * N + v) * N + args.anchors[ac + t]) * tiles_per_view_dev(args.H, args.W) +
+                                         p0 / kTileTokens;
+                        r0 = record_offset(args.tile_ptr, i, args.max_records);
+                        r1 = record_offset(args.tile_ptr, i + 1, args.max_records);
+                    }
+                    s_r0[t] = r0;
+                    s_rn[t] = r1 - r0;
+                }
 #pragma unroll
-            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
-                m[s2] = 0;
-                if (s2 < na && fg)
-                    m[s2] = MODE == GEOCACHE_CORR_MASK
-                                ? __ldg(args.keep + (((size_t)b * N + v) * N + args.anchors[ac + s2]) * plane + p)
-                                : 15u;
-            }
+                for (int s2 = 0; s2 < kTokenAnchors; ++s2) s_has[s2][t] = 0;
+                __syncthreads();
+                int total = 0;
 #pragma unroll
-            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
-                kept[s2] = __ballot_sync(0xffffffffu, m[s2] & 15u);
-                mine += __popc(kept[s2]);
-                s_has[s2][t] = 0;
-            }
-            if (lane == 0) s_wcnt[warp] = mine;
-            __syncthreads();
-            int at = 0, n_items = 0;
-#pragma unroll
-            for (int w = 0; w < kThreads / 32; ++w) {
-                at += w < warp ? s_wcnt[w] : 0;
-                n_items += s_wcnt[w];
-            }
-#pragma unroll
-            for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
-                if (m[s2] & 15u)
-                    s_item[at + __popc(kept[s2] & ((1u << lane) - 1u))] =
-                        (uint32_t)t | ((uint32_t)s2 << 10) | ((m[s2] & 15u) << 16);
-                at += __popc(kept[s2]);
-            }
-            __syncthreads();
-            for (int j = t; j < n_items; j += kThreads) {
-                const uint32_t it = s_item[j];
-                const int lp = (int)(it & 1023u), s2 = (int)((it >> 10) & 63u);
-                Taps tp;
-                item_taps<K, MODE>(args, s_cam[s2], b, v, ac + s2, p0 + lp, (int)(it >> 16), tv0, plane, tau2, tp);
-                if (tp.kept) {
+                for (int s2 = 0; s2 < kTokenAnchors; ++s2) total += s_rn[s2];
+                for (int j = t; j < total; j += kThreads) {
+                    int s2 = 0, jj = j;
+                    while (jj >= s_rn[s2]) jj -= s_rn[s2++];
+                    const int4 rec = __ldg(reinterpret_cast<const int4*>(args.records) + s_r0[s2] + jj);
+                    const int lp = (rec.x & 0x0fffffff) - p0;
+                    if ((unsigned)lp >= (unsigned)kThreads) continue;
+                    Taps tp;
+                    taps_from_record<K>((int)((uint32_t)rec.x >> 28), rec.y, __int_as_float(rec.z),
+                                        __int_as_float(rec.w), args.W, tp);
                     float g[4];
                     item_increment<K>(args, tp, b, ac + s2, cg, cn, plane, g);
                     s_g[s2][lp] = make_float4(g[0], g[1], g[2], g[3]);
                     s_has[s2][lp] = 1;
                 }
+                __syncthreads();
+            } else {
+                if (MODE != GEOCACHE_CORR_TABLE && t < na * 16)
+                    reinterpret_cast<float*>(s_cam)[t] = __ldg(
+                        reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (t >> 4)]) + (t & 15));
+                // the round's candidate (anchor, token)s, listed by warp
+                uint32_t m[kTokenAnchors], kept[kTokenAnchors];
+                int mine = 0;
+#pragma unroll
+                for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                    m[s2] = 0;
+                    if (s2 < na && fg)
+                        m[s2] = MODE == GEOCACHE_CORR_MASK
+                                    ? __ldg(args.keep + (((size_t)b * N + v) * N + args.anchors[ac + s2]) * plane + p)
+                                    : 15u;
+                }
+#pragma unroll
+                for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                    kept[s2] = __ballot_sync(0xffffffffu, m[s2] & 15u);
+                    mine += __popc(kept[s2]);
+                    s_has[s2][t] = 0;
+                }
+                if (lane == 0) s_wcnt[warp] = mine;
+                __syncthreads();
+                int at = 0, n_items = 0;
+#pragma unroll
+                for (int w = 0; w < kThreads / 32; ++w) {
+                    at += w < warp ? s_wcnt[w] : 0;
+                    n_items += s_wcnt[w];
+                }
+#pragma unroll
+                for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
+                    if (m[s2] & 15u)
+                        s_item[at + __popc(kept[s2] & ((1u << lane) - 1u))] =
+                            (uint32_t)t | ((uint32_t)s2 << 10) | ((m[s2] & 15u) << 16);
+                    at += __popc(kept[s2]);
+                }
+                __syncthreads();
+                for (int j = t; j < n_items; j += kThreads) {
+                    const uint32_t it = s_item[j];
+                    const int lp = (int)(it & 1023u), s2 = (int)((it >> 10) & 63u);
+                    Taps tp;
+                    item_taps<K, MODE>(args, s_cam[s2], b, v, ac + s2, p0 + lp, (int)(it >> 16), tv0, plane, tau2, tp);
+                    if (tp.kept) {
+                        float g[4];
+                        item_increment<K>(args, tp, b, ac + s2, cg, cn, plane, g);
+                        s_g[s2][lp] = make_float4(g[0], g[1], g[2], g[3]);
+                        s_has[s2][lp] = 1;
+                    }
+                }
+                __syncthreads();
             }
-            __syncthreads();
 #pragma unroll
             for (int s2 = 0; s2 < kTokenAnchors; ++s2) {
                 if (!s_has[s2][t]) continue;
@@ -1984,15 +2031,6 @@ struct SparseGrid {
     int small;  // n_total * n_stream < 2^31: the interleave's quotients in 32 bits
     FastDiv cg, tiles, a, na, slices, total;
 };
-
-// Tile offset i of the sparse form clamped to the records that exist, [0,
-// cap]: a build whose records overflowed the capacity or the int32 offsets
-// is flagged in the status word, and the transport then reads only records
-// that exist.
-__device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_ptr, size_t i, long long cap) {
-    const long long x = __ldg(tile_ptr + i);
-    return (int)(x < 0 ? 0 : (x < cap ? x : cap));
-}
 
 // Records of one pair applied by one CTA slice (grid-stride over the pair's
 // records), channels [cg, cg + 4).  COPY: the value-copy ablation (no x0(t-1)
@@ -2450,6 +2488,19 @@ constexpr int kSrcMinChannels = 8;
 // many records each, from the mean records per ordered view pair.
 constexpr long long kApplyRecords = 384;
 
+template <typename T, int K, int MODE>
+static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s);
+
+// Units (tiles of 1024 tokens x channel groups) up to which a sparse step that
+// is not in place takes one token per thread from the records, in one launch
+// instead of two and without the workspace rows (us, two launches and one;
+// bf16, 4 channels unless said): 24 units 6.6 and 4.1, 54 9.1 and 5.9, 96 8.9
+// and 5.4 (16 channels 6.8 and 4.5), 200 (f32, 6 channels, 75 x 53) 7.3 and 5.8,
+// 288 10.8 and 8.4, 384 11.4 and 10.5, 432 (12 views, 16 channels) 17.5 and 14.7,
+// but 768 14.1 and 21.2.  (In place the anchors' rows wait for every gather, so a
+// second launch is needed anyway.)
+constexpr long long kTokenUnitsSparse = 384;
+
 template <typename T, int K>
 static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
     const int HW = t.H * t.W;
@@ -2460,6 +2511,8 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
     const bool vec = (HW % 4 == 0) && (al % 16 == 0);
     const bool in_place = t.x0_out == t.x0_prev;
     const bool copy = t.update == GEOCACHE_UPDATE_COPY;
+    if (!in_place && t.a < t.N && (long long)t.B * t.N * n_tiles * n_cg <= kTokenUnitsSparse)
+        return launch_token<T, K, GEOCACHE_CORR_SPARSE>(t, s);
     // wide latents: the anchors' increment plane when the workspace holds it
     // beside max_records * C floats, else phase A by source tile when the
     // corr has a source index and the staged span (tile + W + 1 tokens)

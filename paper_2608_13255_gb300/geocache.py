@@ -517,10 +517,11 @@ def rotate_anchors(N: int, a: int, step: int, S: int, sched: dict):
 
 
 def transport_launches(a: int, N: int, mode: int, in_place: bool = False) -> int:
-    """Kernels one geocache_transport_step enqueues: sparse mode runs the
-    record-parallel apply (when some view is outside the anchor set) and the
-    streaming kernel; the other modes one fused kernel, plus the anchor-row
-    copy of an in-place update."""
+    """Kernels one geocache_transport_step enqueues for a large batch: sparse mode
+    runs the record-parallel apply (when some view is outside the anchor set)
+    and the streaming kernel (small steps that are not in place: one kernel);
+    the other modes one fused kernel, plus the anchor-row copy of an in-place
+    update."""
     if mode == CORR_SPARSE:
         return 2 if a < N else 1
     return 1 + (1 if in_place else 0)

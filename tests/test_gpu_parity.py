@@ -695,6 +695,57 @@ def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
     assert_bf16_close(outs["plane"][1].view(np.uint16), ref_xn, what="x_next")
 
 
+@pytest.mark.parametrize("B,N,H,W,C,a,K,dtype,update,drop", [
+    (32, 6, 32, 32, 8, 2, 4, "bf16", "delta", 0),     # 384 units: the last step of one token per thread
+    (33, 6, 32, 32, 8, 2, 4, "bf16", "copy", 0),      # 396 units: the first of two launches
+    (16, 6, 37, 29, 18, 3, 4, "bf16", "delta", 0),    # unaligned rows, a channel group of 2
+    (16, 6, 48, 40, 16, 5, 1, "f32", "copy", 0),
+    (40, 6, 37, 29, 16, 2, 4, "f32", "delta", 37),    # records beyond the capacity dropped
+    (80, 6, 40, 32, 4, 2, 4, "bf16", "delta", 11),    # few channels
+    (4, 6, 40, 32, 4, 2, 4, "bf16", "delta", 11),     # the same with one token per thread
+])
+def test_sparse_paths_of_large_steps_agree_bitwise(gc, B, N, H, W, C, a, K, dtype, update, drop):
+    # the increment plane, the source-tile apply and the record-parallel apply of steps too large for one token
+    # per thread, against each asset stepped alone (which is not) on the same records
+    w = synth.replicate_assets(synth.make_workload("batch128", B=3, N=N, H=H, W=W), B)
+    pos, valid, cams = (torch.from_numpy(x).cuda() for x in (w.pos, w.valid, w.cams))
+    c = gc.build_sparse_corr(pos, valid, cams, K=K, source_index=True)
+    k = c._keep
+    R = k["records"].shape[0] - drop
+    gen = torch.Generator("cuda").manual_seed(5)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    anchors = sorted(np.random.default_rng(a).choice(N, a, replace=False).tolist())
+    x0, x_t = rnd(B, N, C, H, W), rnd(B, N, C, H, W).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    x0_new = (x0[:, anchors] + 0.1 * rnd(B, a, C, H, W)).contiguous()
+
+    def step(sl, tile_ptr, records, index=False, minimal=False, in_place=False):
+        n = sl.stop - sl.start
+        h = gc.make_corr(pos[sl], valid[sl], cams[sl], c.tau[sl], K=K, keep=c.keep[sl], tile_ptr=tile_ptr, records=records,
+                         src_ptr=k["src_ptr"] if index else None, src_rec=k["src_rec"][:R] if index else None)
+        prev, xt = x0[sl].clone(), x_t[sl].clone()
+        out, xn = (prev, xt) if in_place else (torch.empty_like(prev), torch.empty_like(xt))
+        pred = torch.empty_like(prev)
+        r = gc.make_recon("ddim", a_t=0.4, a_prev=0.5, pred_kind="v", pred_out=pred)
+        ws = torch.empty(max(4, h.min_workspace_floats(C) if minimal else h.workspace_floats(C)), device="cuda")
+        gc.transport_step(h, anchors, C, x0_new[sl], prev, out, xt, xn, r, workspace=ws, update=update)
+        gc.device_status()
+        return [x.view(torch.uint8) for x in (out, xn, pred)]
+
+    pairs = N * N * gc.tiles_per_view(H, W)
+    alone = [step(slice(b, b + 1), k["tile_ptr"][b * pairs:(b + 1) * pairs + 1].contiguous(), k["records"][:R])
+             for b in range(B)]
+    ref = [torch.cat([o[i] for o in alone]) for i in range(3)]
+    whole = slice(0, B)
+    for index, minimal, in_place in ((False, False, False), (True, True, False), (False, True, False),
+                                     (False, False, True)):
+        if index and (drop or C < 8):
+            continue  # the index of a build whose records all fit
+        got = step(whole, k["tile_ptr"], k["records"][:R], index, minimal, in_place)
+        for x, y in zip(got, ref):
+            assert torch.equal(x, y)
+    assert not torch.equal(ref[0], x0.view(torch.uint8))
+
+
 def test_wide_views_fall_back_to_the_record_parallel_apply(gc):
     # W + 1 > 1024 tokens: the staged span of a source tile would not fit, so a
     # step with a source index and a minimal workspace applies the records
