@@ -538,6 +538,9 @@ class Trajectory:
         launches = 0
         gc.build_corr(self.corr)
         launches += 1 + (1 if (self.corr.idx is not None or self.corr.keep is not None) else 0)
+        tiles = w.B * w.N * gc.tiles_per_view(w.H, w.W)
+        if self.corr.idx is None and self.corr.keep is not None and tiles >= 700:
+            launches += 2  # large builds: the source depths before the masks, their clearing after
         if self.corr.c.mode == gc.CORR_SPARSE:
             launches += 2  # the tile offsets' scan, the records
             if self.corr.c.src_ptr:
@@ -566,6 +569,9 @@ class Trajectory:
         out = self.bufs[0] if cache is not self.bufs[0] else self.bufs[1]
         gc.transport_step(self.corr, anchors, w.C, self.anchor_x0[t], cache, out, self.x, self.x, self.recon[t],
                           workspace=self.workspace)
+        units = w.B * w.N * gc.tiles_per_view(w.H, w.W) * -(-w.C // 4)
+        if self.corr.c.mode == gc.CORR_SPARSE and units <= 384:
+            return out, 1  # small steps that are not in place: one launch
         return out, gc.transport_launches(w.a, w.N, self.corr.c.mode, in_place=False)
 
     def capture(self):
