@@ -1172,6 +1172,37 @@ struct Lat4<__nv_bfloat16> {
     }
 };
 
+// Eight consecutive elements: 32-byte accesses of f32 (sm_100 and later) and 16-byte ones of bf16, not kept
+// in the L1
+__device__ __forceinline__ void load8(const float* p, float (&r)[8]) {
+    asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+                 : "l"(p));
+}
+__device__ __forceinline__ void store8(float* p, const float (&r)[8]) {
+    asm volatile("st.global.L1::no_allocate.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r[0]), "f"(r[1]),
+                 "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&r)[8]) {
+    const uint4 x = __ldcs(reinterpret_cast<const uint4*>(p));
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        r[2 * i] = __uint_as_float(w[i] << 16);
+        r[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&r)[8]) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(r[2 * i], r[2 * i + 1]);
+        w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    __stcs(reinterpret_cast<uint4*>(p), make_uint4(w[0], w[1], w[2], w[3]));
+}
+
 // the anchors' rows stay cached (they are re-read by the gathers)
 __device__ __forceinline__ void f4_load_keep(const float* p, size_t e, int cnt, bool vec, float (&r)[4]) {
     if (vec) {
@@ -2811,6 +2842,36 @@ __global__ void __launch_bounds__(256) reconstruct_kernel(const T* xt, const flo
     }
 }
 
+// The same with eight consecutive elements per thread and no loop, for f32
+// pointers on 32 bytes and bf16 ones on 16: half the memory instructions, and a
+// CTA's loads all issue at once.  64 assets x 6 views at 128 x 128 x 4, bf16, x0
+// stored (302 MB): 48.1 -> 44.5 us, 6.78 TB/s (the copy rate); grid-stride
+// over 16 or 32 CTAs per SM 45.8 and 45.2; 128 assets without the store 61.6 ->
+// 56.8, f32 62.5 -> 59.3.
+template <typename T>
+__global__ void __launch_bounds__(256) reconstruct8_kernel(const T* xt, const float* x0, T* xn, int64_t n,
+                                                           const ReconCoef coef, float* pred_out, float* x0_store) {
+    const int64_t e = 8 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (e + 8 <= n) {
+        float a[8], x[8], y[8], pr[8];
+        load8(x0 + e, a);
+        load8(xt + e, x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = recon_one(coef, x[i], a[i], pr[i]);
+        store8(xn + e, y);
+        if (pred_out) store8(pred_out + e, pr);
+        if (x0_store) store8(x0_store + e, a);
+        return;
+    }
+    for (int64_t i = e; i < n; ++i) {  // the last n % 8 elements
+        const float a = x0[i];
+        float pr;
+        lat_store(xn, i, recon_one(coef, lat_load(xt, i), a, pr));
+        if (pred_out) pred_out[i] = pr;
+        if (x0_store) x0_store[i] = a;
+    }
+}
+
 template <typename T>
 static cudaError_t launch_reconstruct_t(const void* x_t, const float* x0, void* x_next, int64_t n,
                                         const ReconCoef& coef, float* pred_out, float* x0_store, cudaStream_t s) {
@@ -2819,7 +2880,11 @@ static cudaError_t launch_reconstruct_t(const void* x_t, const float* x0, void* 
     const uintptr_t al = (uintptr_t)x_t | (uintptr_t)x0 | (uintptr_t)x_next | (uintptr_t)pred_out | (uintptr_t)x0_store;
     const T* xt = static_cast<const T*>(x_t);
     T* xn = static_cast<T*>(x_next);
-    if (al % 16 == 0)
+    const uintptr_t f32s = (uintptr_t)x0 | (uintptr_t)pred_out | (uintptr_t)x0_store, lats = (uintptr_t)x_t | (uintptr_t)x_next;
+    const int64_t blocks8 = (n + 2047) / 2048;
+    if (f32s % 32 == 0 && lats % (8 * sizeof(T)) == 0 && blocks8 <= 0x7fffffffLL)
+        reconstruct8_kernel<T><<<(unsigned)blocks8, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);
+    else if (al % 16 == 0)
         reconstruct_kernel<T, true><<<(unsigned)blocks, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);
     else
         reconstruct_kernel<T, false><<<(unsigned)blocks, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);

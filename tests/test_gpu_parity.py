@@ -210,6 +210,28 @@ def test_corr_modes_agree_bitwise(gc, workloads, name, K):
     np.testing.assert_array_equal(got_mask, got_tab)
 
 
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 2047, 2048, 2055, 70001])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_reconstruct_remainders_and_alignments_agree_bitwise(gc, n, dtype):
+    # 32-byte (8 elements), 16-byte and scalar accesses by the pointers' alignment; prediction and stored x0 beside
+    gen = torch.Generator("cuda").manual_seed(n)
+    x0, xt = torch.randn(n, generator=gen, device="cuda"), torch.randn(n, generator=gen, device="cuda").to(dtype)
+    outs = []
+    for off in (0, 4, 1):
+        at = lambda t, like: torch.full((n + 24,), 9.0, dtype=like.dtype, device="cuda")[off:off + n] if t is None else \
+            torch.cat([torch.zeros(off, dtype=t.dtype, device="cuda"), t])[off:]
+        a, x = at(x0, None), at(xt, None)
+        xn, pred, store = at(None, xt), at(None, x0), at(None, x0)
+        gc.reconstruct(x, a, xn, gc.make_recon("ddim", a_t=0.3, a_prev=0.4, pred_kind="eps", pred_out=pred), x0_store=store)
+        outs.append((xn, pred, store))
+    for got in outs[1:]:
+        for g, r in zip(got, outs[0]):
+            assert torch.equal(g, r)
+    assert torch.equal(outs[0][2], x0)
+    eps = (xt.double() - math.sqrt(0.3) * x0.double()) / math.sqrt(0.7)
+    assert_f32_close(outs[0][1].cpu().numpy(), eps.cpu().numpy(), scale=1 + math.sqrt(0.3) / math.sqrt(0.7), what="eps")
+
+
 @pytest.mark.parametrize("B,N,H,W,C,a,K,dtype,update,in_place", [
     (1, 6, 16, 16, 4, 2, 4, "bf16", "delta", False),    # one tile of 256 tokens, exactly
     (2, 6, 37, 29, 5, 5, 4, "bf16", "delta", True),     # ragged, two rounds of anchors, a channel group of 1
