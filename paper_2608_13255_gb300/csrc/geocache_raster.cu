@@ -3,7 +3,8 @@
 // (Sec. 3.1), from which the correspondence operator of Sec. 3.2 is built.
 //
 // A z-buffer over pixel centres, in two kernels:
-//  raster_faces_kernel: one thread per face, looping over the views (the
+//  raster_faces_kernel: one thread per face (fewer per warp in small renders of
+//    large faces), looping over the CTA's views (the
 //    face's vertices are loaded once; a CTA's faces normally belong to one
 //    asset, whose cameras are staged in shared memory).  For each view the
 //    face is projected; every pixel centre inside or on it (three
@@ -58,6 +59,13 @@ __device__ unsigned int g_raster_error = 0;
 
 constexpr int kRasterThreads = 256;
 constexpr int kRasterBlocks = 4;  // resident CTAs per SM of the face kernel
+
+// How a render is split over CTAs: `views` consecutive views per CTA (each CTA
+// loads its faces again) and `faces` faces per warp (32 or fewer; all 32 lanes
+// still share the warp's pixels).
+struct RasterSplit {
+    int views, faces;
+};
 constexpr unsigned long long kEmpty = ~0ull;  // z-buffer word of an uncovered pixel
 
 struct Cam32 {
@@ -228,11 +236,11 @@ __device__ __forceinline__ float small_float(int x) { return __int_as_float(x | 
 template <bool ONE>
 __device__ __forceinline__ void raster_warp(const float (&X)[3][3], bool ok, int b, unsigned int f_warp,
                                             const geocache_camera* s_cam, const geocache_camera* __restrict__ cams,
-                                            const int* b_w, WarpFaces& sh, int N, int H, int W,
+                                            const int* b_w, WarpFaces& sh, int N, int view0, int view1, int H, int W,
                                             float scale, unsigned long long* __restrict__ zbuf) {
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
-    for (int view = 0; view < N; ++view) {
+    for (int view = view0; view < view1; ++view) {
         // depth and z-buffer update of the pixel with centre (pu, pv), covered by the face of a slot
         auto resolve = [&](int slot, float pu, float pv) {
             const int src = sh.info[slot].lane;
@@ -323,18 +331,19 @@ __device__ __forceinline__ void raster_warp(const float (&X)[3][3], bool ok, int
 
 __global__ void __launch_bounds__(kRasterThreads, kRasterBlocks) raster_faces_kernel(
     const float* __restrict__ V, long long nv, const int32_t* __restrict__ F, long long nf,
-    const int64_t* __restrict__ face_off, int B, const geocache_camera* __restrict__ cams, int N, int H, int W,
+    const int64_t* __restrict__ face_off, int B, const geocache_camera* __restrict__ cams, int N, RasterSplit split, int H, int W,
     float scale, unsigned long long* __restrict__ zbuf) {
     __shared__ geocache_camera s_cam[GEOCACHE_MAX_VIEWS];
     __shared__ int s_asset[2];
     __shared__ WarpFaces s_faces[kRasterThreads / 32];
     __shared__ int s_b[kRasterThreads];
-    const long long f0 = blockIdx.x * (long long)kRasterThreads;
-    const long long f = f0 + threadIdx.x;
-    const int w0 = threadIdx.x & ~31;
+    const int w0 = threadIdx.x & ~31, lane = threadIdx.x & 31;
+    const int per_cta = split.faces * (kRasterThreads / 32);
+    const long long f0 = blockIdx.x * (long long)per_cta, f_warp = f0 + (w0 >> 5) * split.faces;
+    const long long f = f_warp + lane;
     // the CTA's faces belong to one asset unless it straddles a boundary
     if (threadIdx.x == 0) s_asset[0] = asset_of(face_off, B, f0);
-    if (threadIdx.x == 1) s_asset[1] = asset_of(face_off, B, min(f0 + kRasterThreads, nf) - 1);
+    if (threadIdx.x == 1) s_asset[1] = asset_of(face_off, B, min(f0 + per_cta, nf) - 1);
     __syncthreads();
     const bool one_asset = s_asset[0] == s_asset[1];
     for (int i = threadIdx.x; i < N * 16; i += kRasterThreads) {
@@ -342,7 +351,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterBlocks) raster_faces_ke
         reinterpret_cast<float*>(s_cam)[i] = (i & 15) >= 12 ? __fmul_rn(x, scale) : x;  // fx, fy, cx, cy
     }
     int b = s_asset[0];
-    bool ok = f < nf;
+    bool ok = lane < split.faces && f < nf;
     float X[3][3];
     if (ok) {
         if (!one_asset) b = asset_of(face_off, B, f);
@@ -361,10 +370,14 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterBlocks) raster_faces_ke
     }
     s_b[threadIdx.x] = b;
     __syncthreads();
+    // the CTA's views
+    const int view0 = blockIdx.y * split.views, view1 = min(view0 + split.views, N);
     if (one_asset)
-        raster_warp<true>(X, ok, b, (unsigned int)(f0 + w0), s_cam, cams, s_b + w0, s_faces[w0 >> 5], N, H, W, scale, zbuf);
+        raster_warp<true>(X, ok, b, (unsigned int)f_warp, s_cam, cams, s_b + w0, s_faces[w0 >> 5], N,
+                          view0, view1, H, W, scale, zbuf);
     else
-        raster_warp<false>(X, ok, b, (unsigned int)(f0 + w0), s_cam, cams, s_b + w0, s_faces[w0 >> 5], N, H, W, scale, zbuf);
+        raster_warp<false>(X, ok, b, (unsigned int)f_warp, s_cam, cams, s_b + w0, s_faces[w0 >> 5], N,
+                          view0, view1, H, W, scale, zbuf);
 }
 
 // World position of the surface point of pixel (i, j) whose z-buffer key is
@@ -579,13 +592,42 @@ cudaError_t read_raster_error(unsigned int* out, bool clear, cudaStream_t s) {
     return cudaStreamSynchronize(s);
 }
 
-// grid of a grid-stride kernel over n items: at most 16 CTAs per SM
-static unsigned stride_grid(long long n) {
+static int sm_count() {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = (n + kRasterThreads - 1) / kRasterThreads, cap = (long long)(sms > 0 ? sms : 1) * 16;
+    return sms > 0 ? sms : 1;
+}
+
+// grid of a grid-stride kernel over n items: at most 16 CTAs per SM
+static unsigned stride_grid(long long n) {
+    const long long want = (n + kRasterThreads - 1) / kRasterThreads, cap = (long long)sm_count() * 16;
     return (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
+}
+
+// All views and 32 faces per warp where that fills the GPU.  A render of more
+// pixels per view than faces per asset is bound by its boxes' pixels: its views
+// are split until there are 4 waves of CTAs, then its faces until there are 4
+// again or a warp's faces hold about kRasterWarpPixels of a view's pixels.
+// One of small faces is bound by loading them, which each CTA does again for
+// its views: it fills one wave only.  Calls, us, unsplit and split: one mesh x 6
+// views of 1,280 faces at 512 x 512 718 and 38 (views alone 137; 512 and 1024
+// pixels a warp 36 and 47, but two such meshes at 160 x 160 19 and 26 against
+// 16), of 20,480 at 288 x 288 90 and 35, of 5,120 at 64 x 64 19 and 8; 3 x 8
+// views of 81,920 at 296 x 512 278 and 240; one x 6 of 81,920 at 128 x 128 19
+// and (views split) 23, so those stay whole.
+constexpr long long kRasterWarpPixels = 256;
+
+static RasterSplit raster_split(long long nf, int B, int N, long long n_pix) {
+    const long long slots = (long long)kRasterBlocks * sm_count(), gx = (nf + kRasterThreads - 1) / kRasterThreads;
+    const bool heavy = n_pix * B > nf;
+    long long chunks = heavy ? (4 * slots + gx - 1) / gx : slots / gx;
+    chunks = chunks < 1 ? 1 : (chunks > N ? N : chunks);
+    RasterSplit split{(int)((N + chunks - 1) / chunks), 32};
+    while (heavy && split.views == 1 && split.faces > 1 && n_pix * B / nf * split.faces > kRasterWarpPixels &&
+           gx * N * (32 / split.faces) < 4 * slots)
+        split.faces /= 2;
+    return split;
 }
 
 cudaError_t launch_raster(const float* V, long long nv, const int32_t* F, long long nf, const int64_t* face_off,
@@ -595,10 +637,11 @@ cudaError_t launch_raster(const float* V, long long nv, const int32_t* F, long l
     cudaError_t e = cudaMemsetAsync(zbuf, 0xff, sizeof(unsigned long long) * (size_t)n_pix, s);
     if (e != cudaSuccess) return e;
     if (nf > 0) {
-        const long long gx = (nf + kRasterThreads - 1) / kRasterThreads;
+        const RasterSplit split = raster_split(nf, B, N, (long long)H * W * ss * ss);
+        const long long per_cta = split.faces * (kRasterThreads / 32), gx = (nf + per_cta - 1) / per_cta;
         if (gx > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        raster_faces_kernel<<<(unsigned)gx, kRasterThreads, 0, s>>>(V, nv, F, nf, face_off, B, cams, N, H * ss,
-                                                                    W * ss, (float)ss, zbuf);
+        raster_faces_kernel<<<dim3((unsigned)gx, (unsigned)((N + split.views - 1) / split.views)), kRasterThreads, 0, s>>>(
+            V, nv, F, nf, face_off, B, cams, N, split, H * ss, W * ss, (float)ss, zbuf);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -99,6 +99,27 @@ def test_box_sizes_bit_exact(gc, kind, H, W):
     assert ref_v.any()
 
 
+@pytest.mark.parametrize("faces,s", [(0, 1), (1, 1), (7, 2), (33, 1), (130, 4), (900, 1)])
+def test_split_renders_bit_exact(gc, faces, s):
+    # few faces of many pixels: the views and the faces of a warp are split over CTAs (down to one face per warp), with
+    # assets changing inside a CTA and a warp
+    H, W = 40, 52
+    views = synth.ring_layout(7, 20.0)
+    cams = np.stack([np.stack([synth.look_at_camera(az, el, H, W) for az, el in views])] * 3)
+    rng = np.random.default_rng(faces + s)
+    meshes = []
+    for n in (faces, 0, max(1, faces // 3)):
+        V = (rng.uniform(-0.6, 0.6, (n, 1, 3)) + 0.5 * rng.standard_normal((n, 3, 3))).reshape(-1, 3).astype(np.float32)
+        meshes.append((V, np.arange(3 * n, dtype=np.int32).reshape(-1, 3)))
+    pos, valid = gc.raster_posmaps(*_upload(meshes, cams), H, W, s=s)
+    torch.cuda.synchronize()
+    gc.device_status()
+    for b, (V, F) in enumerate(meshes):
+        ref_p, ref_v = oracle.raster_supersampled(V, F, cams[b], H, W, s)
+        np.testing.assert_array_equal(valid.cpu().numpy()[b], ref_v)
+        np.testing.assert_array_equal(pos.cpu().numpy()[b].view(np.uint32), ref_p.view(np.uint32))
+
+
 def test_posmaps_feed_the_correspondence_build(gc):
     # the rasterised maps of a blob are a valid input of the correspondence
     # build, which then gives the oracle's tables
