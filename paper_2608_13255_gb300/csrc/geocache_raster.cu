@@ -26,7 +26,7 @@
 //    differences stored with the face, without a branch; and the three IEEE
 //    divisions of a depth run with full warps (with one lane in eight when
 //    each warp formed the depths as it met them).  16 meshes x 6 views at
-//    128 x 128: 454 -> 253 us; 4 smooth ones at 512 x 512: 134 -> 87 us.
+//    128 x 128: 454 -> 241 us; 4 smooth ones at 512 x 512: 134 -> 83 us.
 //    4 resident CTAs per SM (64 registers); 3, 5 and 6: 6%, 9% and 20%
 //    slower.
 //  raster_resolve_kernel: one thread per pixel; the key's depth gives the
@@ -150,9 +150,10 @@ __device__ __forceinline__ void ray(const Cam32& c, float pu, float pv, float& d
 // Faces of a warp published for its pixel loop: 20 words each, so that eight
 // different faces read by 16-byte loads fall into different banks.
 //   [0..2]  edge k = 0, 1, 2 from vertex a to vertex b ((1,2), (2,0), (0,1)):
-//           (u_b - u_a, v_b - v_a) and (u_a, v_a)
+//           (u_b - u_a, v_b - v_a), both negated when the area is negative
+//           (which negates the edge function exactly), and (u_a, v_a)
 //   [3]     first pixel of the face in the warp's concatenated boxes,
-//           1 / box width (negative: the area is), centre of the box's first pixel
+//           1 / box width (to an ulp), centre of the box's first pixel
 //   [4]     n, nd
 // and beside them (SlotInfo) the box width and the face's lane.
 constexpr int kSlotQuads = 5;
@@ -165,10 +166,11 @@ __device__ __forceinline__ void publish_face(float4* q, SlotInfo* info, const Fa
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int a = (k + 1) % 3, b = (k + 2) % 3;
-        q[k] = make_float4(__fsub_rn(o.u[b], o.u[a]), __fsub_rn(o.v[b], o.v[a]), o.u[a], o.v[a]);
+        const float du = __fsub_rn(o.u[b], o.u[a]), dv = __fsub_rn(o.v[b], o.v[a]);
+        q[k] = make_float4(o.area < 0.0f ? -du : du, o.area < 0.0f ? -dv : dv, o.u[a], o.v[a]);
     }
-    const float width = o.ihi - o.ilo + 1.0f, inv = __frcp_rn(width);
-    q[3] = make_float4(__int_as_float(start), o.area < 0.0f ? -inv : inv, o.ilo + 0.5f, o.jlo + 0.5f);
+    const float width = o.ihi - o.ilo + 1.0f;
+    q[3] = make_float4(__int_as_float(start), __fdividef(1.0f, width), o.ilo + 0.5f, o.jlo + 0.5f);
     q[4] = make_float4(o.n[0], o.n[1], o.n[2], o.nd);
     *info = SlotInfo{width, lane};
 }
@@ -176,15 +178,13 @@ __device__ __forceinline__ void publish_face(float4* q, SlotInfo* info, const Fa
 // whether the centre (pu, pv) lies inside or on the published face: its three
 // edge functions (u_b - u_a)(pv - v_a) - (v_b - v_a)(pu - u_a) have the sign
 // of the area or are zero
-__device__ __forceinline__ bool covers(const float4* q, bool negative, float pu, float pv) {
+__device__ __forceinline__ bool covers(const float4* q, float pu, float pv) {
     const float4 e[3] = {q[0], q[1], q[2]};
     float w[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         w[k] = __fsub_rn(__fmul_rn(e[k].x, __fsub_rn(pv, e[k].w)), __fmul_rn(e[k].y, __fsub_rn(pu, e[k].z)));
-    const bool up = (w[0] >= 0.0f) & (w[1] >= 0.0f) & (w[2] >= 0.0f);
-    const bool down = (w[0] <= 0.0f) & (w[1] <= 0.0f) & (w[2] <= 0.0f);
-    return negative ? down : up;
+    return (w[0] >= 0.0f) & (w[1] >= 0.0f) & (w[2] >= 0.0f);
 }
 
 // depth key of the covered pixel with centre (pu, pv), or kEmpty when the ray
@@ -281,12 +281,12 @@ __device__ __forceinline__ void raster_warp(const float (&X)[3][3], bool ok, int
             const float4* q = sh.slot + slot * kSlotQuads;
             const float4 h = q[3];
             const float local = small_float(k - __float_as_int(h.x));
-            // row of the box: local / width by the reciprocal, exact since the box has at most
-            // 2^16 pixels (the quotient is at least 0.5 / width from an integer); rounding the sum
-            // with 2^23 down leaves its integer part
-            const float row = __fadd_rd((local + 0.5f) * fabsf(h.y), kTwo23) - kTwo23;
+            // row of the box: local / width by the reciprocal, exact since the box has at most 2^16
+            // pixels (the quotient is at least 0.5 / width from an integer, its error below 2^-4 /
+            // width); rounding the sum with 2^23 down leaves its integer part
+            const float row = __fadd_rd((local + 0.5f) * h.y, kTwo23) - kTwo23;
             const float pu = h.z + __fmaf_rn(-row, sh.info[slot].width, local), pv = h.w + row;
-            const bool in = covers(q, h.y < 0.0f, pu, pv) & (k0 + lane < total);
+            const bool in = covers(q, pu, pv) & (k0 + lane < total);
             const uint32_t hits = __ballot_sync(0xffffffffu, in);
             if (in) {
                 const int at = n_queued + __popc(hits & below);
@@ -320,10 +320,9 @@ __device__ __forceinline__ void raster_warp(const float (&X)[3][3], bool ok, int
             const float ilo = __shfl_sync(0xffffffffu, o.ilo, src), ihi = __shfl_sync(0xffffffffu, o.ihi, src);
             const float jlo = __shfl_sync(0xffffffffu, o.jlo, src), jhi = __shfl_sync(0xffffffffu, o.jhi, src);
             __syncwarp();
-            const bool negative = sh.slot[3].y < 0.0f;
             for (float j = jlo; j <= jhi; j += 1.0f)
                 for (float i = ilo + (float)lane; i <= ihi; i += 32.0f)
-                    if (covers(sh.slot, negative, i + 0.5f, j + 0.5f)) resolve(0, i + 0.5f, j + 0.5f);
+                    if (covers(sh.slot, i + 0.5f, j + 0.5f)) resolve(0, i + 0.5f, j + 0.5f);
             __syncwarp();
         }
     }
