@@ -66,6 +66,8 @@ typedef enum {
     GEOCACHE_CORR_MASK = 2,     /* read the 1-byte keep masks written by geocache_build_corr; recompute
                                    the projection and weights only where a tap is kept */
     GEOCACHE_CORR_SPARSE = 3    /* read the sparse tap records written by geocache_build_corr (fastest):
+                                   small steps that are not in place apply them in one kernel, without
+                                   the workspace; otherwise:
                                    C < 8, or a workspace without room for the increment plane: the
                                    records are applied record-parallel (or per source tile with a
                                    source index) into workspace rows; C >= 8 with room: the anchors'

@@ -229,18 +229,22 @@ static_assert(GEOCACHE_TILE_TOKENS % kBuildThreads == 0, "a build CTA's tokens l
 // the source loop (the background is ~60% of a view).  REP = 4 for large
 // builds with tables (large builds without take build_keep_kernel), 1 for
 // small ones, where the 4x fewer CTAs would not fill the GPU.
-template <int K, bool TABLES, int REP>
+template <int K, bool TABLES, int REP, bool SPLIT>
 __global__ void __launch_bounds__(kBuildThreads) build_corr_kernel(const float* __restrict__ pos,
                                                          const uint8_t* __restrict__ valid,
                                                          const geocache_camera* __restrict__ cams,
                                                          const float* __restrict__ tau, int N, int H, int W,
                                                          int32_t* __restrict__ idx, float* __restrict__ wout,
-                                                         uint8_t* __restrict__ keep, int32_t* __restrict__ tile_cnt) {
+                                                         uint8_t* __restrict__ keep, int32_t* __restrict__ tile_cnt,
+                                                         int n_split) {
     static_assert(GEOCACHE_TILE_TOKENS % (kBuildThreads * REP) == 0, "a build CTA's tokens lie in one tile");
     const int HW = H * W;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int p_base = blockIdx.x * kBuildThreads * REP;
-    const int v = blockIdx.y, b = blockIdx.z;
+    // SPLIT: n_split CTAs share the source views of the same tokens
+    const int v = SPLIT ? blockIdx.y / n_split : blockIdx.y, b = blockIdx.z;
+    const int part = SPLIT ? (int)blockIdx.y - v * n_split : 0;
+    const int u_first = SPLIT ? part * N / n_split : 0, u_last = SPLIT ? (part + 1) * N / n_split : N;
     __shared__ geocache_camera s_cam[GEOCACHE_MAX_VIEWS];
     __shared__ int s_fg[kBuildThreads * REP];
     __shared__ int s_wcnt[REP][kBuildThreads / 32];
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_corr_kernel(const float* 
             X1 = __ldg(pos + 3 * (view0 + pw) + 1);
             X2 = __ldg(pos + 3 * (view0 + pw) + 2);
         }
-        for (int u = 0; u < N; ++u) {
+        for (int u = u_first; u < u_last; ++u) {
             Taps tp;
             taps_clear(tp);
             int mask = 0;
@@ -592,12 +596,24 @@ __global__ void __launch_bounds__(256) clear_diagonal_kernel(uint8_t* keep, int 
     clear_chunk(row, HW, blockIdx.x * 256 + threadIdx.x);
 }
 
+// CTAs from which a build's CTAs take all source views of their tokens.  With
+// fewer, a CTA's views in sequence are the time of the kernel: one asset of 6
+// views at 64 x 64 (96 CTAs) 7.5 us, with its views split over 576 CTAs 4.3; 4
+// views at 96 x 96 (144) 5.4 and 4.0, 8 at 64 x 64 (128) 9.5 and 5.7.  From 384 CTAs (6 views at 128 x 128)
+// on the split gains nothing (8.6 and 8.3), beyond 608 it loses.
+constexpr long long kBuildCtas = 608;
+
 template <int K, bool TABLES, int REP>
 static void launch_build_corr_rep(const geocache_corr& c, int32_t* cnt, cudaStream_t s) {
-    const int HW = c.H * c.W;
-    const dim3 grid((HW + kBuildThreads * REP - 1) / (kBuildThreads * REP), c.N, c.B);
-    build_corr_kernel<K, TABLES, REP><<<grid, kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx,
-                                                                     c.w, c.keep, cnt);
+    const int HW = c.H * c.W, gx = (HW + kBuildThreads * REP - 1) / (kBuildThreads * REP);
+    const long long ctas = (long long)gx * c.N * c.B, want = (kBuildCtas + ctas - 1) / ctas;
+    const int n_split = (int)(want < c.N ? want : c.N);
+    if (REP == 1 && n_split > 1)
+        build_corr_kernel<K, TABLES, 1, true><<<dim3(gx, c.N * n_split, c.B), kBuildThreads, 0, s>>>(
+            c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx, c.w, c.keep, cnt, n_split);
+    else
+        build_corr_kernel<K, TABLES, REP, false><<<dim3(gx, c.N, c.B), kBuildThreads, 0, s>>>(
+            c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx, c.w, c.keep, cnt, 1);
 }
 
 // Tiles from which the depth test pays for its two extra launches and its
