@@ -17,6 +17,12 @@
 
 namespace geocache {
 
+// Programmatic dependent launch: the dependent grid may start once every CTA
+// of this grid has issued launch_dependents (or ended); griddepcontrol.wait
+// blocks until the grids before it have completed and their writes are visible.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 struct Taps {
     int32_t q[4];   // source token index row*W + col, -1 = not kept
     float w[4];     // renormalised weight, 0 where not kept

@@ -99,6 +99,26 @@ cudaError_t launch_raster(const float* V, long long nv, const int32_t* F, long l
 cudaError_t launch_pool_posmaps(const float* pos_hi, const uint8_t* valid_hi, long long n_maps, int H, int W, int ss,
                                 float* pos, uint8_t* valid, cudaStream_t s);
 
+// Launch with programmatic stream serialization: the kernel may become resident
+// while the one before it in the stream drains, and begins with pdl_wait, before
+// it touches memory.  It hides the launch behind the predecessor's tail (a call,
+// among others of its kind: 128 assets' cached step 111.0 -> 108.4 us, 8 assets
+// of 12 views x 16 channels 77.6 -> 74.6).
+template <typename... Params, typename... Args>
+cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, size_t dyn_smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = dyn_smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+
 // Records a status and its message for geocache_last_error(); returns status.
 int set_error(int status, const char* fmt, ...);
 

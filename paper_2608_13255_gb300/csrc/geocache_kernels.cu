@@ -1757,6 +1757,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
     __shared__ geocache_camera s_cam[kTokenAnchors];
     __shared__ int s_wcnt[kThreads / 32];
     __shared__ int s_r0[kTokenAnchors], s_rn[kTokenAnchors];  // SPARSE: the tile's records of the round's anchors
+    pdl_wait();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int HW = args.H * args.W, N = args.N, C = args.C, a = args.a;
     const size_t plane = (size_t)HW;
@@ -2065,13 +2066,6 @@ struct QuadRows {
     }
 };
 
-// Programmatic dependent launch: the dependent grid may start once every CTA
-// of this grid has issued launch_dependents; griddepcontrol.wait blocks until
-// the prerequisite grid has completed and its writes are visible.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-
 // Grid shape of a sparse step's launches and the divisors that split it.
 struct SparseGrid {
     int n_cg, n_tiles, n_slices, n_stream, n_total;
@@ -2166,6 +2160,7 @@ constexpr int kPlaneBBlocks = 5;
 template <typename T, int K, bool VEC, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_kernel(const TransportArgs args,
                                                                                     const SparseGrid g) {
+    pdl_wait();  // launched while the kernel before it drains: everything it wrote is visible from here
     pdl_launch_dependents();
     const uint32_t k = blockIdx.x;
     int s_before, s_next;
@@ -2212,6 +2207,7 @@ __global__ void __launch_bounds__(kThreads, PK ? kPlaneBBlocks : kPhaseBBlocks<T
     __shared__ float s_acc[kTileTokens][4];
     __shared__ __align__(4) uint8_t s_n[kTileTokens];
     __shared__ int s_r0[GEOCACHE_MAX_VIEWS], s_cnt[GEOCACHE_MAX_VIEWS];
+    if (PK) pdl_launch_dependents();  // the next step's phase A may take the places of this grid's last CTAs
     const int HW = args.H * args.W;
     const int T_tiles = tiles_per_view_dev(args.H, args.W);
     const int n_cg = g.n_cg;
@@ -2352,6 +2348,7 @@ __global__ void __launch_bounds__(kThreads, PK ? kPlaneBBlocks : kPhaseBBlocks<T
 template <typename T, bool VEC, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPlaneABlocks) sparse_phase_a_plane_kernel(const TransportArgs args,
                                                                                          const SparseGrid g) {
+    pdl_wait();  // launched while the kernel before it drains: everything it wrote is visible from here
     pdl_launch_dependents();
     const int HW = args.H * args.W;
     const int n_cg = g.n_cg;
@@ -2421,6 +2418,7 @@ __global__ void __launch_bounds__(kThreads, kPlaneABlocks) sparse_phase_a_plane_
 template <typename T, int K, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_src_kernel(const TransportArgs args,
                                                                                        const SparseGrid g, int stream) {
+    pdl_wait();  // launched while the kernel before it drains: everything it wrote is visible from here
     pdl_launch_dependents();
     extern __shared__ __align__(16) float4 s_d[];  // [kTileTokens + W + 1] tokens x 4 channels
     const int HW = args.H * args.W, W = args.W;
@@ -2580,22 +2578,21 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
     if (by_plane) {
         const long long g = (long long)t.B * t.a * n_tiles * n_cg;
         if (g > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        if (vec && !copy) sparse_phase_a_plane_kernel<T, true, false><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
-        else if (vec) sparse_phase_a_plane_kernel<T, true, true><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
-        else if (!copy) sparse_phase_a_plane_kernel<T, false, false><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
-        else sparse_phase_a_plane_kernel<T, false, true><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
-        cudaError_t e = cudaGetLastError();
+        const dim3 grid((unsigned)g);
+        cudaError_t e = vec ? (copy ? launch_pdl(sparse_phase_a_plane_kernel<T, true, true>, grid, kThreads, 0, s, t, sg)
+                                    : launch_pdl(sparse_phase_a_plane_kernel<T, true, false>, grid, kThreads, 0, s, t, sg))
+                            : (copy ? launch_pdl(sparse_phase_a_plane_kernel<T, false, true>, grid, kThreads, 0, s, t, sg)
+                                    : launch_pdl(sparse_phase_a_plane_kernel<T, false, false>, grid, kThreads, 0, s, t, sg));
         if (e != cudaSuccess) return e;
         phase_a = true;
     } else if (by_source) {
         const long long g = (long long)t.B * t.a * n_tiles * n_cg;
         if (g > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         const size_t dyn = (size_t)(kTileTokens + t.W + 1) * sizeof(float4);
-        if (!copy)
-            sparse_phase_a_src_kernel<T, K, false><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
-        else
-            sparse_phase_a_src_kernel<T, K, true><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
-        cudaError_t e = cudaGetLastError();
+        const dim3 grid((unsigned)g);
+        const int stream = in_place ? 0 : 1;
+        cudaError_t e = copy ? launch_pdl(sparse_phase_a_src_kernel<T, K, true>, grid, kThreads, dyn, s, t, sg, stream)
+                             : launch_pdl(sparse_phase_a_src_kernel<T, K, false>, grid, kThreads, dyn, s, t, sg, stream);
         if (e != cudaSuccess) return e;
         phase_a = true;
     } else {
@@ -2615,15 +2612,10 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
             sg.n_total = (int)g;
             sg.total = make_fastdiv(g);
             sg.small = (long long)g * n_stream < 0x80000000LL;
-            if (vec && !copy)
-                sparse_phase_a_kernel<T, K, true, false><<<g, kThreads, 0, s>>>(t, sg);
-            else if (vec)
-                sparse_phase_a_kernel<T, K, true, true><<<g, kThreads, 0, s>>>(t, sg);
-            else if (!copy)
-                sparse_phase_a_kernel<T, K, false, false><<<g, kThreads, 0, s>>>(t, sg);
-            else
-                sparse_phase_a_kernel<T, K, false, true><<<g, kThreads, 0, s>>>(t, sg);
-            cudaError_t e = cudaGetLastError();
+            cudaError_t e = vec ? (copy ? launch_pdl(sparse_phase_a_kernel<T, K, true, true>, dim3(g), kThreads, 0, s, t, sg)
+                                        : launch_pdl(sparse_phase_a_kernel<T, K, true, false>, dim3(g), kThreads, 0, s, t, sg))
+                                : (copy ? launch_pdl(sparse_phase_a_kernel<T, K, false, true>, dim3(g), kThreads, 0, s, t, sg)
+                                        : launch_pdl(sparse_phase_a_kernel<T, K, false, false>, dim3(g), kThreads, 0, s, t, sg));
             if (e != cudaSuccess) return e;
             phase_a = true;
         }
@@ -2681,8 +2673,7 @@ template <typename T, int K, int MODE>
 static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s) {
     const int HW = t.H * t.W, n_cg = (t.C + 3) / 4;
     const dim3 grid((unsigned)((HW + kThreads - 1) / kThreads * n_cg), t.N, t.B);
-    transport_token_kernel<T, K, MODE><<<grid, kThreads, 0, s>>>(t, make_fastdiv((uint32_t)n_cg));
-    return cudaGetLastError();
+    return launch_pdl(transport_token_kernel<T, K, MODE>, grid, kThreads, 0, s, t, make_fastdiv((uint32_t)n_cg));
 }
 
 template <typename T, int K>
@@ -2867,6 +2858,7 @@ __global__ void __launch_bounds__(256) reconstruct_kernel(const T* xt, const flo
 template <typename T>
 __global__ void __launch_bounds__(256) reconstruct8_kernel(const T* xt, const float* x0, T* xn, int64_t n,
                                                            const ReconCoef coef, float* pred_out, float* x0_store) {
+    pdl_wait();
     const int64_t e = 8 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (e + 8 <= n) {
         float a[8], x[8], y[8], pr[8];
@@ -2899,8 +2891,8 @@ static cudaError_t launch_reconstruct_t(const void* x_t, const float* x0, void* 
     const uintptr_t f32s = (uintptr_t)x0 | (uintptr_t)pred_out | (uintptr_t)x0_store, lats = (uintptr_t)x_t | (uintptr_t)x_next;
     const int64_t blocks8 = (n + 2047) / 2048;
     if (f32s % 32 == 0 && lats % (8 * sizeof(T)) == 0 && blocks8 <= 0x7fffffffLL)
-        reconstruct8_kernel<T><<<(unsigned)blocks8, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);
-    else if (al % 16 == 0)
+        return launch_pdl(reconstruct8_kernel<T>, dim3((unsigned)blocks8), 256, 0, s, xt, x0, xn, n, coef, pred_out, x0_store);
+    if (al % 16 == 0)
         reconstruct_kernel<T, true><<<(unsigned)blocks, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);
     else
         reconstruct_kernel<T, false><<<(unsigned)blocks, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);

@@ -46,6 +46,7 @@
 #include <cstdint>
 
 #include "geocache.h"
+#include "geocache_device.cuh"
 #include "geocache_internal.h"
 
 namespace geocache {
@@ -512,6 +513,7 @@ __global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const floa
                                                                        int H, int W, int s, long long n_tok,
                                                                        float* __restrict__ pos,
                                                                        uint8_t* __restrict__ valid) {
+    pdl_wait();
     const long long HW = (long long)H * W;
     const long long Ws = (long long)W * s;
     for (long long p = blockIdx.x * (long long)kRasterThreads + threadIdx.x; p < n_tok;
@@ -670,8 +672,7 @@ cudaError_t launch_pool_posmaps(const float* pos_hi, const uint8_t* valid_hi, lo
         else if (ss == 4) kern = pool_posmaps_kernel<4>;
         else if (ss == 8) kern = pool_posmaps_kernel<8>;
     }
-    kern<<<stride_grid(n_tok), kRasterThreads, 0, s>>>(pos_hi, valid_hi, H, W, ss, n_tok, pos, valid);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(stride_grid(n_tok)), kRasterThreads, 0, s, pos_hi, valid_hi, H, W, ss, n_tok, pos, valid);
 }
 
 }  // namespace geocache
