@@ -88,7 +88,8 @@ def test_tables_bit_exact_k1(gc, workloads, name):
 
 
 @pytest.mark.parametrize("H,W,B,K,scene", [(24, 21, 320, 4, "plain"), (24, 21, 320, 1, "plain"), (37, 29, 160, 4, "far"),
-                                           (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd")])
+                                           (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd"),
+                                           (37, 29, 1900, 4, "plain")])  # 136,800 counts: two rounds of the scan
 def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
     # builds of at least 700 tiles test a source depth before the taps, and fill their records with a warp per tile
     # from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
