@@ -637,7 +637,8 @@ cudaError_t launch_build_corr(const geocache_corr& c, cudaStream_t s) {
         else
             build_keep_kernel<1><<<dim3(T, c.N, c.B), kBuildThreads, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N, c.H,
                                                                              c.W, c.keep, c.tile_ptr);
-        clear_diagonal_kernel<<<dim3((unsigned)(HW / 4096 + 1), c.N, c.B), 256, 0, s>>>(c.keep, c.N, HW);
+        const int chunks = HW / 16 + 2;  // of a row that starts anywhere in a 16-byte word (clear_chunk)
+        clear_diagonal_kernel<<<dim3((unsigned)((chunks + 255) / 256), c.N, c.B), 256, 0, s>>>(c.keep, c.N, HW);
         return cudaGetLastError();
     }
     int32_t* cnt = nullptr;

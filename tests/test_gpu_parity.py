@@ -89,12 +89,15 @@ def test_tables_bit_exact_k1(gc, workloads, name):
 
 @pytest.mark.parametrize("H,W,B,K,scene", [(24, 21, 320, 4, "plain"), (24, 21, 320, 1, "plain"), (37, 29, 160, 4, "far"),
                                            (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd"),
-                                           (37, 29, 1900, 4, "plain")])  # 136,800 counts: two rounds of the scan
+                                           (37, 29, 1900, 4, "plain"),  # 136,800 counts: two rounds of the scan
+                                           (63, 65, 30, 4, "plain"), (63, 65, 30, 1, "offset"),
+                                           (126, 130, 8, 4, "plain"), (40, 32, 160, 4, "offset")])
 def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
     # builds of at least 700 tiles test a source depth before the taps, and fill their records with a warp per tile
     # from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
     # that the oracle checks).  far: an asset 3,000 units from the origin (the depths' rounding); scaled: cameras with
-    # rows of other lengths than 1; odd: infinite, huge and NaN positions, and an empty asset
+    # rows of other lengths than 1; odd: infinite, huge and NaN positions, and an empty asset; offset: masks 1 byte off
+    # their alignment (rows of 4,095 and 16,380 tokens begin anywhere in a 16-byte word: the diagonal's last bytes)
     w = synth.make_workload("batch128", B=6, H=H, W=W)
     w.pos, w.cams = w.pos.copy(), w.cams.copy()
     R, t = w.cams[..., :9].reshape(6, w.N, 3, 3), w.cams[..., 9:12]
@@ -112,10 +115,13 @@ def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
     big = synth.replicate_assets(w, B)
     d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
     c = gc.build_sparse_corr(d(big.pos), d(big.valid), d(big.cams), K=K)
-    keep = torch.full((B, w.N, w.N, H, W), 77, dtype=torch.uint8, device="cuda")
+    skew = 1 if scene == "offset" else 0
+    keep = torch.full((skew + B * w.N * w.N * H * W,), 77, dtype=torch.uint8, device="cuda")[skew:]
+    keep = keep.view(B, w.N, w.N, H, W)
     gc.build_corr(gc.make_corr(d(big.pos), d(big.valid), d(big.cams), torch.zeros(B, device="cuda"), K=K, keep=keep))
     whole = gc.build_corr(c)  # masks, offsets and records in one call
     gc.device_status()
+    assert int(torch.diagonal(keep, dim1=1, dim2=2).count_nonzero()) == 0
     assert torch.equal(keep, c.keep)
     T, pairs = gc.tiles_per_view(H, W), w.N * w.N
     ptr, rec = whole._keep["tile_ptr"], whole._keep["records"]
