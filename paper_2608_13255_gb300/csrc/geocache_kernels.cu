@@ -363,7 +363,10 @@ __global__ void __launch_bounds__(kBuildThreads) build_corr_kernel(const float* 
 // z + 1e-6 S of its foreground texels plus |R2| tau (1 + 1e-5) and the change of
 // S over a distance tau; -inf without foreground.  It covers 9 x 9 texels: the
 // block and the column and row after it, so that one value serves every
-// footprint whose top-left tap lies in the block.  A NaN never rejects.
+// footprint whose top-left tap lies in the block.  A NaN never rejects, and
+// nothing is rejected where a square underflows: with tau^2 or |R2|^2 below
+// 1e-30 the tap test's distances (then of few or no bits) or |R2| say nothing
+// about the depths.
 //
 // The values lie in the keep masks' diagonal rows (u = v), which hold no masks
 // and are cleared after the build, so that no scratch is needed.
@@ -435,8 +438,10 @@ __global__ void __launch_bounds__(256) source_depth_kernel(const float* __restri
     const int bx = (x0 + lane) / kDepthBlock;
     if (lane % kDepthBlock == 0 && bx < nbx) {
         const float t = __ldg(tau + b);
-        const float norm2 = sqrtf(r0 * r0 + r1 * r1 + r2 * r2), norm1 = fabsf(r0) + fabsf(r1) + fabsf(r2);
-        depth_row(keep, view, v, N, HW)[by * nbx + bx] = block + t * (1.00001f * norm2 + 1e-6f * norm1);
+        const float sq = r0 * r0 + r1 * r1 + r2 * r2, norm2 = sqrtf(sq), norm1 = fabsf(r0) + fabsf(r1) + fabsf(r2);
+        const bool bounded = t * t >= 1e-30f && sq >= 1e-30f;
+        depth_row(keep, view, v, N, HW)[by * nbx + bx] =
+            bounded ? block + t * (1.00001f * norm2 + 1e-6f * norm1) : INFINITY;
     }
 }
 

@@ -91,13 +91,15 @@ def test_tables_bit_exact_k1(gc, workloads, name):
                                            (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd"),
                                            (37, 29, 1900, 4, "plain"),  # 136,800 counts: two rounds of the scan
                                            (63, 65, 30, 4, "plain"), (63, 65, 30, 1, "offset"),
-                                           (126, 130, 8, 4, "plain"), (40, 32, 160, 4, "offset")])
+                                           (126, 130, 8, 4, "plain"), (40, 32, 160, 4, "offset"),
+                                           (40, 32, 160, 4, "minute"), (40, 32, 160, 4, "faint")])
 def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
     # builds of at least 700 tiles test a source depth before the taps, and fill their records with a warp per tile
     # from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
     # that the oracle checks).  far: an asset 3,000 units from the origin (the depths' rounding); scaled: cameras with
-    # rows of other lengths than 1; odd: infinite, huge and NaN positions, and an empty asset; offset: masks 1 byte off
-    # their alignment (rows of 4,095 and 16,380 tokens begin anywhere in a 16-byte word: the diagonal's last bytes)
+    # rows of other lengths than 1; faint and minute: rows, and positions, whose squares underflow; odd: infinite, huge
+    # and NaN positions, and an empty asset; offset: masks 1 byte off their alignment (rows of 4,095 and 16,380 tokens
+    # begin anywhere in a 16-byte word: the diagonal's last bytes)
     w = synth.make_workload("batch128", B=6, H=H, W=W)
     w.pos, w.cams = w.pos.copy(), w.cams.copy()
     R, t = w.cams[..., :9].reshape(6, w.N, 3, 3), w.cams[..., 9:12]
@@ -105,8 +107,11 @@ def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
         shift = np.array([3000.0, -1500.0, 800.0])
         w.cams[..., 9:12] = t - (R.astype(np.float64) @ shift)
         w.pos = (w.pos.astype(np.float64) + shift).astype(np.float32)
-    if scene == "scaled":
-        w.cams[..., :12] *= np.float32(3.7)
+    if scene in ("scaled", "faint"):
+        w.cams[..., :12] *= np.float32(3.7 if scene == "scaled" else 1e-25)
+    if scene == "minute":
+        w.pos *= np.float32(1e-22)
+        w.cams[..., 9:12] *= np.float32(1e-22)
     if scene == "odd":
         fg = np.argwhere(w.valid[:3] > 0)
         for k, x in enumerate((np.inf, 3e38, np.nan, 1e20, -np.inf)):
