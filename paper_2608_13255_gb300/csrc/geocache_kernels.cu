@@ -1927,6 +1927,13 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
 //    increments in anchor order (deterministic: the mean over covering
 //    anchors of Eq. 1 with the aggregation of Sec. 3.2; tokens without a
 //    record keep x0(t-1)), then stores and reconstructs every token.
+// Phase B becomes resident while phase A drains and reads tile_ptr and its
+// streamed rows (x0(t-1), x_t) before it waits; CTAs of tiles without records
+// never wait.  Phase A writes none of these, and it is launched in stream
+// order, after everything before it has completed, so they are written and
+// visible before either phase starts.  (Phase A launched early too, with all of
+// phase B waiting: 128 assets 112.3 us against 111.1, 8 assets of 12 views x 16
+// channels 77.8 against 78.3.)
 // Wide latents (C >= 8) with room in the workspace take another phase A:
 // the anchor views streamed while their increments are written once as a
 // plane (4 channels per 16-byte word), from which phase B forms each
@@ -2166,10 +2173,6 @@ constexpr int kPlaneBBlocks = 5;
 template <typename T, int K, bool VEC, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_kernel(const TransportArgs args,
                                                                                     const SparseGrid g) {
-    pdl_wait();  // launched while the kernel before it drains (launch_pdl)
-    // phase B, some of whose CTAs do not wait, may start only now that this grid's predecessors have completed.  (Phase
-    // B itself does not trigger: the next step's CTAs, waiting beside it, took 128 assets from 108.8 to 112.1 us and one
-    // asset of 12 views x 16 channels from 15.2 to 16.7.)
     pdl_launch_dependents();
     const uint32_t k = blockIdx.x;
     int s_before, s_next;
@@ -2356,7 +2359,6 @@ __global__ void __launch_bounds__(kThreads, PK ? kPlaneBBlocks : kPhaseBBlocks<T
 template <typename T, bool VEC, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPlaneABlocks) sparse_phase_a_plane_kernel(const TransportArgs args,
                                                                                          const SparseGrid g) {
-    pdl_wait();  // launched while the kernel before it drains (launch_pdl)
     pdl_launch_dependents();
     const int HW = args.H * args.W;
     const int n_cg = g.n_cg;
@@ -2426,7 +2428,6 @@ __global__ void __launch_bounds__(kThreads, kPlaneABlocks) sparse_phase_a_plane_
 template <typename T, int K, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_src_kernel(const TransportArgs args,
                                                                                        const SparseGrid g, int stream) {
-    pdl_wait();  // launched while the kernel before it drains (launch_pdl)
     pdl_launch_dependents();
     extern __shared__ __align__(16) float4 s_d[];  // [kTileTokens + W + 1] tokens x 4 channels
     const int HW = args.H * args.W, W = args.W;
@@ -2586,21 +2587,22 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
     if (by_plane) {
         const long long g = (long long)t.B * t.a * n_tiles * n_cg;
         if (g > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        const dim3 grid((unsigned)g);
-        cudaError_t e = vec ? (copy ? launch_pdl(sparse_phase_a_plane_kernel<T, true, true>, grid, kThreads, 0, s, t, sg)
-                                    : launch_pdl(sparse_phase_a_plane_kernel<T, true, false>, grid, kThreads, 0, s, t, sg))
-                            : (copy ? launch_pdl(sparse_phase_a_plane_kernel<T, false, true>, grid, kThreads, 0, s, t, sg)
-                                    : launch_pdl(sparse_phase_a_plane_kernel<T, false, false>, grid, kThreads, 0, s, t, sg));
+        if (vec && !copy) sparse_phase_a_plane_kernel<T, true, false><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
+        else if (vec) sparse_phase_a_plane_kernel<T, true, true><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
+        else if (!copy) sparse_phase_a_plane_kernel<T, false, false><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
+        else sparse_phase_a_plane_kernel<T, false, true><<<(unsigned)g, kThreads, 0, s>>>(t, sg);
+        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         phase_a = true;
     } else if (by_source) {
         const long long g = (long long)t.B * t.a * n_tiles * n_cg;
         if (g > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         const size_t dyn = (size_t)(kTileTokens + t.W + 1) * sizeof(float4);
-        const dim3 grid((unsigned)g);
-        const int stream = in_place ? 0 : 1;
-        cudaError_t e = copy ? launch_pdl(sparse_phase_a_src_kernel<T, K, true>, grid, kThreads, dyn, s, t, sg, stream)
-                             : launch_pdl(sparse_phase_a_src_kernel<T, K, false>, grid, kThreads, dyn, s, t, sg, stream);
+        if (!copy)
+            sparse_phase_a_src_kernel<T, K, false><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
+        else
+            sparse_phase_a_src_kernel<T, K, true><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
+        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         phase_a = true;
     } else {
@@ -2620,10 +2622,15 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
             sg.n_total = (int)g;
             sg.total = make_fastdiv(g);
             sg.small = (long long)g * n_stream < 0x80000000LL;
-            cudaError_t e = vec ? (copy ? launch_pdl(sparse_phase_a_kernel<T, K, true, true>, dim3(g), kThreads, 0, s, t, sg)
-                                        : launch_pdl(sparse_phase_a_kernel<T, K, true, false>, dim3(g), kThreads, 0, s, t, sg))
-                                : (copy ? launch_pdl(sparse_phase_a_kernel<T, K, false, true>, dim3(g), kThreads, 0, s, t, sg)
-                                        : launch_pdl(sparse_phase_a_kernel<T, K, false, false>, dim3(g), kThreads, 0, s, t, sg));
+            if (vec && !copy)
+                sparse_phase_a_kernel<T, K, true, false><<<g, kThreads, 0, s>>>(t, sg);
+            else if (vec)
+                sparse_phase_a_kernel<T, K, true, true><<<g, kThreads, 0, s>>>(t, sg);
+            else if (!copy)
+                sparse_phase_a_kernel<T, K, false, false><<<g, kThreads, 0, s>>>(t, sg);
+            else
+                sparse_phase_a_kernel<T, K, false, true><<<g, kThreads, 0, s>>>(t, sg);
+            cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             phase_a = true;
         }
