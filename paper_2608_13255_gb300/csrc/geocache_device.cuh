@@ -55,10 +55,11 @@ __device__ __forceinline__ bool project(const geocache_camera& c, float X0, floa
     return true;
 }
 
+// (coherent loads: a GEOMETRY step is launched while what writes the maps may still run)
 __device__ __forceinline__ float sqdist(const float* P, float X0, float X1, float X2) {
-    const float dx = __fsub_rn(__ldg(P + 0), X0);
-    const float dy = __fsub_rn(__ldg(P + 1), X1);
-    const float dz = __fsub_rn(__ldg(P + 2), X2);
+    const float dx = __fsub_rn(__ldca(P + 0), X0);
+    const float dy = __fsub_rn(__ldca(P + 1), X1);
+    const float dz = __fsub_rn(__ldca(P + 2), X2);
     return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
@@ -120,7 +121,7 @@ __device__ __forceinline__ int tap_mask(const Footprint& f, const float* __restr
         if (col < 0 || col >= W || row < 0 || row >= H) continue;
         if (K == 4 && (f.ax[di] == 0.0f || f.ay[dj] == 0.0f)) continue;
         const int q = row * W + col;
-        const int fg = __ldg(valid_u + q) != 0;
+        const int fg = __ldca(valid_u + q) != 0;
         const int near = sqdist(pos_u + 3 * (size_t)q, X0, X1, X2) <= tau2;
         mask |= (fg & near) << k;
     }

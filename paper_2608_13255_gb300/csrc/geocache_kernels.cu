@@ -17,8 +17,13 @@ namespace geocache {
 
 __host__ __device__ int tiles_per_view(int H, int W) { return (H * W + GEOCACHE_TILE_TOKENS - 1) / GEOCACHE_TILE_TOKENS; }
 
+// Loads: __ldg (ld.global.nc) is for memory that nothing writes while the kernel
+// is resident.  A kernel launched early (launch_pdl, phase B) is resident before
+// the kernel that writes its inputs has ended, and an in-place step writes rows
+// that it reads; those load by __ldca or __ldcs, which are coherent.
+
 // ---------------------------------------------------------------- latents --
-__device__ __forceinline__ float lat_load(const float* p, size_t i) { return __ldg(p + i); }
+__device__ __forceinline__ float lat_load(const float* p, size_t i) { return __ldca(p + i); }
 __device__ __forceinline__ float lat_load(const __nv_bfloat16* p, size_t i) {
     return __bfloat162float(p[i]);
 }
@@ -1365,8 +1370,8 @@ __device__ __forceinline__ void item_taps(const TransportArgs& args, const geoca
         tp.kept = 0;
 #pragma unroll
         for (int kk = 0; kk < K; ++kk) {
-            int q = __ldg(args.idx + row * K + kk);
-            float wq = __ldg(args.w + row * K + kk);
+            int q = __ldca(args.idx + row * K + kk);
+            float wq = __ldca(args.w + row * K + kk);
             if (q < -1 || q >= (int)plane) {  // a caller's table with an index outside the view: dropped, reported
                 atomicOr(&g_device_error, 16u);
                 q = -1;
@@ -1378,9 +1383,9 @@ __device__ __forceinline__ void item_taps(const TransportArgs& args, const geoca
         }
         return;
     }
-    const float X0 = __ldg(args.pos + 3 * (tv0 + p));
-    const float X1 = __ldg(args.pos + 3 * (tv0 + p) + 1);
-    const float X2 = __ldg(args.pos + 3 * (tv0 + p) + 2);
+    const float X0 = __ldca(args.pos + 3 * (tv0 + p));
+    const float X1 = __ldca(args.pos + 3 * (tv0 + p) + 1);
+    const float X2 = __ldca(args.pos + 3 * (tv0 + p) + 2);
     if (MODE == GEOCACHE_CORR_MASK) {
         Footprint f;
         footprint<K>(cam, X0, X1, X2, args.H, args.W, f);
@@ -1408,8 +1413,8 @@ __device__ __forceinline__ void item_increment(const TransportArgs& args, const 
             dp[kk][c] = 0.0f;
             if (tp.q[kk] >= 0 && c < cn) {
                 const size_t e = (size_t)c * plane + tp.q[kk];
-                dn[kk][c] = __ldg(xn + e);
-                dp[kk][c] = __ldg(xp + e);
+                dn[kk][c] = __ldca(xn + e);
+                dp[kk][c] = __ldca(xp + e);
             }
         }
 #pragma unroll
@@ -1731,7 +1736,7 @@ static FastDiv make_fastdiv(uint32_t d) {
 // is flagged in the status word, and the transport then reads only records
 // that exist.
 __device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_ptr, size_t i, long long cap) {
-    const long long x = __ldg(tile_ptr + i);
+    const long long x = __ldca(tile_ptr + i);
     return (int)(x < 0 ? 0 : (x < cap ? x : cap));
 }
 
@@ -1780,17 +1785,17 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
     float x0[4], xt[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        x0[c] = in && c < cn ? __ldg(src + (size_t)c * plane) : 0.0f;
+        x0[c] = in && c < cn ? __ldca(src + (size_t)c * plane) : 0.0f;
         xt[c] = in && c < cn && recon ? lat_load(xt_p, base + (size_t)c * plane) : 0.0f;
     }
     if (slot < 0) {
         const size_t tv0 = ((size_t)b * N + v) * plane;
         float tau2 = 0.0f;
         if (MODE == GEOCACHE_CORR_GEOMETRY) {
-            const float tu = __ldg(args.tau + b);
+            const float tu = __ldca(args.tau + b);
             tau2 = __fmul_rn(tu, tu);
         }
-        const bool fg = in && (MODE != GEOCACHE_CORR_GEOMETRY || __ldg(args.valid + tv0 + p) != 0);
+        const bool fg = in && (MODE != GEOCACHE_CORR_GEOMETRY || __ldca(args.valid + tv0 + p) != 0);
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         int n = 0;
         for (int ac = 0; ac < a; ac += kTokenAnchors) {
@@ -1818,7 +1823,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
                 for (int j = t; j < total; j += kThreads) {
                     int s2 = 0, jj = j;
                     while (jj >= s_rn[s2]) jj -= s_rn[s2++];
-                    const int4 rec = __ldg(reinterpret_cast<const int4*>(args.records) + s_r0[s2] + jj);
+                    const int4 rec = __ldca(reinterpret_cast<const int4*>(args.records) + s_r0[s2] + jj);
                     const int lp = (rec.x & 0x0fffffff) - p0;
                     if ((unsigned)lp >= (unsigned)kThreads) continue;
                     Taps tp;
@@ -1832,7 +1837,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
                 __syncthreads();
             } else {
                 if (MODE != GEOCACHE_CORR_TABLE && t < na * 16)
-                    reinterpret_cast<float*>(s_cam)[t] = __ldg(
+                    reinterpret_cast<float*>(s_cam)[t] = __ldca(
                         reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (t >> 4)]) + (t & 15));
                 // the round's candidate (anchor, token)s, listed by warp
                 uint32_t m[kTokenAnchors], kept[kTokenAnchors];
@@ -1842,7 +1847,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
                     m[s2] = 0;
                     if (s2 < na && fg)
                         m[s2] = MODE == GEOCACHE_CORR_MASK
-                                    ? __ldg(args.keep + (((size_t)b * N + v) * N + args.anchors[ac + s2]) * plane + p)
+                                    ? __ldca(args.keep + (((size_t)b * N + v) * N + args.anchors[ac + s2]) * plane + p)
                                     : 15u;
                 }
 #pragma unroll
@@ -2298,7 +2303,7 @@ __global__ void __launch_bounds__(kThreads, PK ? kPlaneBBlocks : kPhaseBBlocks<T
                 float4 dq[PK ? PK : 1];
 #pragma unroll
                 for (int kk = 0; kk < (PK ? PK : 1); ++kk)
-                    dq[kk] = tp.q[kk] >= 0 ? __ldg(d + tp.q[kk]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    dq[kk] = tp.q[kk] >= 0 ? __ldca(d + tp.q[kk]) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int kk = 0; kk < (PK ? PK : 1); ++kk) {
                     if (tp.q[kk] < 0) continue;

@@ -506,10 +506,12 @@ __global__ void __launch_bounds__(kRasterThreads) raster_pool_kernel(const unsig
 // With S a token's row comes as one word of validity and 8- or 16-byte words of
 // positions (scalar loads at s = 8 touch each
 // 128-byte line 32 times): 96 maps of 512 x 512 to 64 x 64, 63.8 -> 33.2
-// us (332 MB, of which the rows without foreground are not read).
+// us (332 MB, of which the rows without foreground are not read).  Launched while
+// the kernel that writes the fine maps may still run, so its loads are coherent
+// ones after the wait.
 template <int S>
-__global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const float* __restrict__ pos_hi,
-                                                                       const uint8_t* __restrict__ valid_hi,
+__global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const float* pos_hi,
+                                                                       const uint8_t* valid_hi,
                                                                        int H, int W, int s, long long n_tok,
                                                                        float* __restrict__ pos,
                                                                        uint8_t* __restrict__ valid) {
@@ -529,12 +531,12 @@ __global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const floa
             for (int sy = 0; sy < S; ++sy) {
                 const uint8_t* v = valid_hi + q0 + sy * Ws;
                 if (S == 8) {
-                    const uint2 w = __ldg(reinterpret_cast<const uint2*>(v));
+                    const uint2 w = __ldca(reinterpret_cast<const uint2*>(v));
                     m[sy][0] = w.x;
                     m[sy][S > 4 ? 1 : 0] = w.y;
                 } else {
-                    m[sy][0] = S == 4 ? __ldg(reinterpret_cast<const uint32_t*>(v))
-                                      : (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(v));
+                    m[sy][0] = S == 4 ? __ldca(reinterpret_cast<const uint32_t*>(v))
+                                      : (uint32_t)__ldca(reinterpret_cast<const unsigned short*>(v));
                 }
             }
 #pragma unroll
@@ -545,7 +547,7 @@ __global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const floa
                 if (S == 2) {
 #pragma unroll
                     for (int h = 0; h < 3 * S / 2; ++h) {
-                        const float2 w = any ? __ldg(reinterpret_cast<const float2*>(row) + h) : make_float2(0.f, 0.f);
+                        const float2 w = any ? __ldca(reinterpret_cast<const float2*>(row) + h) : make_float2(0.f, 0.f);
                         x[2 * h] = w.x;
                         x[2 * h + 1] = w.y;
                     }
@@ -553,7 +555,7 @@ __global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const floa
 #pragma unroll
                     for (int h = 0; h < 3 * S / 4; ++h) {
                         const float4 w =
-                            any ? __ldg(reinterpret_cast<const float4*>(row) + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            any ? __ldca(reinterpret_cast<const float4*>(row) + h) : make_float4(0.f, 0.f, 0.f, 0.f);
                         x[4 * h] = w.x;
                         x[4 * h + 1] = w.y;
                         x[4 * h + 2] = w.z;
@@ -571,8 +573,8 @@ __global__ void __launch_bounds__(kRasterThreads) pool_posmaps_kernel(const floa
             for (int sy = 0; sy < s; ++sy)
                 for (int sx = 0; sx < s; ++sx) {
                     const long long q = base + ((long long)j * s + sy) * Ws + (long long)i * s + sx;
-                    if (!__ldg(valid_hi + q)) continue;
-                    const float X[3] = {__ldg(pos_hi + 3 * q), __ldg(pos_hi + 3 * q + 1), __ldg(pos_hi + 3 * q + 2)};
+                    if (!__ldca(valid_hi + q)) continue;
+                    const float X[3] = {__ldca(pos_hi + 3 * q), __ldca(pos_hi + 3 * q + 1), __ldca(pos_hi + 3 * q + 2)};
                     acc.add(X);
                 }
         }
