@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import operator
 import os
 
 import torch
@@ -306,7 +307,7 @@ _SCHED_KINDS = {"every_k": SCHED_EVERY_K, "head_mid_tail": SCHED_HEAD_MID_TAIL, 
 def _schedule_values(spec: dict):
     get = spec.get
     return (_SCHED_KINDS[spec["kind"]], int(get("k", 1)), int(get("head", 2)), int(get("mid", 1)),
-            int(get("tail", 1)), tuple(get("steps", ())), int(get("contiguous", 0)))
+            int(get("tail", 1)), tuple(map(operator.index, get("steps", ()))), int(get("contiguous", 0)))
 
 
 def _make_schedule(kind, k, head, mid, tail, steps, contiguous):

@@ -56,6 +56,21 @@ def test_schedule_matches_oracle(gc, sched):
             assert gc.is_full_step(t, S, sched) == oracle.is_full_step(t, S, sched), (t, S)
 
 
+def test_full_steps_that_are_not_integers_are_refused(gc):
+    # equal in value to a schedule asked about before, and refused like before
+    for steps in ([0, 3, 7], [0.0, 3.0, 7.0], [0, 3, 7], [0.0, 3.0, 7.0]):
+        sched = {"kind": "list", "steps": steps}
+        if isinstance(steps[0], int):
+            assert gc.is_full_step(3, 10, sched) and gc.rotate_anchors(6, 2, 3, 10, sched)[1]
+            continue
+        with pytest.raises(TypeError):
+            gc.is_full_step(3, 10, sched)
+        with pytest.raises(TypeError):
+            gc.rotate_anchors(6, 2, 3, 10, sched)
+        with pytest.raises(TypeError):
+            gc.make_schedule(sched)
+
+
 @pytest.mark.parametrize("N,a", [(6, 2), (6, 3), (12, 4), (10, 2), (6, 4), (7, 3), (6, 6), (6, 1)])
 def test_rotation_matches_oracle(gc, N, a):
     sched = {"kind": "every_k", "k": 5}
