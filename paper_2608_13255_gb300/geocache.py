@@ -341,7 +341,6 @@ def transport_step(corr: CorrHandle, anchors, C, x0_anchor_new, x0_prev, x0_out,
     c = corr.c
     anc = sorted(map(int, anchors))
     a = len(anc)
-    C = int(C)
     per = C * c.H * c.W
     n_anc, n_all = c.B * a * per, c.B * c.N * per
     arr = (ctypes.c_int32 * max(1, a))(*anc)
@@ -355,7 +354,7 @@ def transport_step(corr: CorrHandle, anchors, C, x0_anchor_new, x0_prev, x0_out,
         r = ctypes.byref(recon)
     f32 = torch.float32
     _check(load().geocache_transport_step_update(
-        ctypes.byref(c), UPDATES[update], arr, a, C, _dev(x0_anchor_new, f32, n_anc, "x0_anchor_new"),
+        ctypes.byref(c), UPDATES[update], arr, a, int(C), _dev(x0_anchor_new, f32, n_anc, "x0_anchor_new"),
         _dev(x0_prev, f32, n_all, "x0_prev"), _dev(x0_out, f32, n_all, "x0_out"), pt, pn, lat, r,
         _dev(workspace, f32, None, "workspace"), 0 if workspace is None else workspace.numel(), _stream(stream)))
 

@@ -282,6 +282,16 @@ def test_mode_kernels_agree_bitwise(gc, B, N, H, W, C, a, K, dtype, update, in_p
             assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
 
 
+def test_channel_count_must_match_the_tensors(gc, workloads):
+    w = workloads("tiny")
+    g = DeviceGeometry(w, K=4, tables=False)
+    x0 = torch.zeros((w.B, w.N, w.C, w.H, w.W), device="cuda")
+    for C in (w.C + 0.5, w.C + 1):  # 0.5: its integer part is the tensors'
+        for step in (gc.transport_step, gc.transport_step_noalloc):
+            with pytest.raises(ValueError):
+                step(g.corr, [0, 3], C, x0[:, :2].contiguous(), x0, torch.empty_like(x0))
+
+
 @pytest.mark.parametrize("pred", ["eps", "v"])
 def test_ddim_prediction_outputs(gc, workloads, pred):
     w = workloads("hunyuan64")
