@@ -2550,15 +2550,25 @@ constexpr long long kApplyRecords = 384;
 template <typename T, int K, int MODE>
 static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s);
 
-// Units (tiles of 1024 tokens x channel groups) up to which a sparse step that
-// is not in place takes one token per thread from the records, in one launch
-// instead of two and without the workspace rows (us, two launches and one;
-// bf16, 4 channels unless said): 24 units 6.6 and 4.1, 54 9.1 and 5.9, 96 8.9
-// and 5.4 (16 channels 6.8 and 4.5), 200 (f32, 6 channels, 75 x 53) 7.3 and 5.8,
-// 288 10.8 and 8.4, 384 11.4 and 10.5, 432 (12 views, 16 channels) 17.5 and 14.7,
-// but 768 14.1 and 21.2.  (In place the anchors' rows wait for every gather, so a
-// second launch is needed anyway.)
-constexpr long long kTokenUnitsSparse = 384;
+// A sparse step that is not in place takes one token per thread from the records,
+// in one launch instead of two and without the workspace, up to kTokenUnitsSparse
+// units (tiles of 1024 tokens x channel groups; in place the anchors' rows wait
+// for every gather, so a second launch is needed anyway).  Its cost grows with
+// the units of the target views, whose CTAs each read the records of the whole
+// tile around their 256 tokens, so those have a lower limit of their own, by what
+// the two launches would do: gather from the increment plane, or apply the
+// records into rows, or that with unaligned rows.  Device us of the two launches
+// and the one (bf16; a anchors of 6 views unless said):
+//   plane     64 x 64 x 8, a = 1: 80 target units 5.6 and 4.0, 160 5.8 and 6.3, 240 6.3
+//             and 7.7; a = 4: 96 9.9 and 7.5, 128 10.2 and 8.8; 24 views of 32 x 32 x 8,
+//             a = 4: 120 8.4 and 9.5
+//   rows      64 x 64 x 4, a = 2: 160 8.0 and 7.3, 192 8.2 and 8.1, 256 8.4 and 9.9; 12
+//             views, a = 4: 192 15.9 and 12.3
+//   unaligned 75 x 53 x 4: a = 1, 240: 9.7 and 8.1, 320 10.5 and 10.0, 480 11.1 and 13.6
+// Over 760 steps of up to 384 units (6 to 64 views of 16 x 16 to 128 x 128, 1 to 48
+// anchors) the limits choose within 1% of the faster on average, 23% at worst;
+// 384 units alone 7% and 86%.
+constexpr long long kTokenUnitsSparse = 384, kTokenTargetsPlane = 144, kTokenTargetsRows = 256, kTokenTargetsUnaligned = 320;
 
 template <typename T, int K>
 static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
@@ -2570,8 +2580,6 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
     const bool vec = (HW % 4 == 0) && (al % 16 == 0);
     const bool in_place = t.x0_out == t.x0_prev;
     const bool copy = t.update == GEOCACHE_UPDATE_COPY;
-    if (!in_place && t.a < t.N && (long long)t.B * t.N * n_tiles * n_cg <= kTokenUnitsSparse)
-        return launch_token<T, K, GEOCACHE_CORR_SPARSE>(t, s);
     // wide latents: the anchors' increment plane when the workspace holds it
     // beside max_records * C floats, else phase A by source tile when the
     // corr has a source index and the staged span (tile + W + 1 tokens)
@@ -2588,6 +2596,10 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
                           t.workspace_floats >= t.max_records * (long long)t.C + n_plane;
     const bool by_source = !by_plane && t.a < t.N && t.src_ptr && t.src_rec && t.C >= kSrcMinChannels &&
                            t.W + 1 <= kTileTokens;
+    const long long per_view = (long long)t.B * n_tiles * n_cg;
+    if (!in_place && t.a < t.N && per_view * t.N <= kTokenUnitsSparse &&
+        per_view * (t.N - t.a) <= (!vec ? kTokenTargetsUnaligned : (by_plane ? kTokenTargetsPlane : kTokenTargetsRows)))
+        return launch_token<T, K, GEOCACHE_CORR_SPARSE>(t, s);
     bool phase_a = false;
     if (by_plane) {
         const long long g = (long long)t.B * t.a * n_tiles * n_cg;

@@ -740,8 +740,11 @@ def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
 
 
 @pytest.mark.parametrize("B,N,H,W,C,a,K,dtype,update,drop", [
-    (32, 6, 32, 32, 8, 2, 4, "bf16", "delta", 0),     # 384 units: the last step of one token per thread
-    (33, 6, 32, 32, 8, 2, 4, "bf16", "copy", 0),      # 396 units: the first of two launches
+    (18, 6, 32, 32, 8, 2, 4, "bf16", "delta", 0),     # 144 units of target views: the last step of one launch
+    (19, 6, 32, 32, 8, 2, 4, "bf16", "copy", 0),      # 152: the first of two (increment plane)
+    (32, 6, 40, 32, 4, 2, 4, "f32", "delta", 0),      # 256: the last of one launch (rows)
+    (33, 6, 40, 32, 4, 2, 4, "f32", "delta", 0),      # 264: the first of two
+    (41, 6, 37, 29, 4, 2, 4, "bf16", "delta", 0),     # 328, unaligned rows: the first of two
     (16, 6, 37, 29, 18, 3, 4, "bf16", "delta", 0),    # unaligned rows, a channel group of 2
     (16, 6, 48, 40, 16, 5, 1, "f32", "copy", 0),
     (40, 6, 37, 29, 16, 2, 4, "f32", "delta", 37),    # records beyond the capacity dropped
