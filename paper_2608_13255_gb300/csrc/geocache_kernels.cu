@@ -2695,11 +2695,18 @@ static int persistent_grid(Kern kern, size_t dyn_smem) {
 }
 
 // Units (tiles of 1024 tokens x channel groups) up to which a MASK step takes
-// one token per thread: with 16-byte aligned rows, against the staged kernel
-// (us; 3 anchors, 96 x 96 x 4 bf16): 24 units 9.0 -> 4.4, 432 19.7 -> 12.0, 864
-// 30.7 -> 28.0, but 1,728 49.1 -> 53.9; otherwise against one CTA per tile
-// (75 x 53 x 4): 96 units 8.2 -> 5.1, 384 11.9 -> 11.1, but 960 23.7 -> 29.2.
-constexpr long long kTokenUnitsStaged = 1024, kTokenUnitsSimple = 384;
+// one token per thread.  With 16-byte aligned rows, against the staged kernel
+// (us; 96 x 96 x 4 bf16, 6 views, 3 anchors): 24 units 8.3 and 4.6, 432 18.7 and
+// 12.7, 1,728 49.1 and 53.9; between 512 and 1,024 units it is the faster for
+// assets of many tokens, with few anchors later (768 units: 6 views of 32 x 32 x 4,
+// 2 anchors 16.0 and 21.2; 12 of 64 x 64 x 4, 4 anchors 37.4 and 26.3).  Otherwise
+// against one CTA per tile (75 x 53 x 4): 96 units 8.2 and 5.1, 384 11.9 and 11.1,
+// 960 23.7 and 29.2.
+static long long mask_token_units(const TransportArgs& t, bool staged) {
+    if (!staged) return 384;
+    const long long asset = (long long)t.N * t.H * t.W;
+    return asset >= (t.a <= 2 ? 98304 : 24576) ? 1024 : 512;
+}
 
 template <typename T, int K, int MODE>
 static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s) {
@@ -2719,7 +2726,7 @@ static cudaError_t launch_mask(const TransportArgs& t, cudaStream_t s) {
     const long long n_units = (long long)t.B * t.N * n_tiles * n_cg;
     const bool staged = vec && HW % 8 == 0;
     // (a pending request of the test hook is for the staged kernel)
-    if (n_units <= (staged ? kTokenUnitsStaged : kTokenUnitsSimple) && !(staged && g_drop_first_copy.load()))
+    if (n_units <= mask_token_units(t, staged) && !(staged && g_drop_first_copy.load()))
         return launch_token<T, K, GEOCACHE_CORR_MASK>(t, s);
     // TMA bulk rows need 16-byte aligned starts and sizes: HW % 8 == 0 covers bf16 rows
     if (staged) {

@@ -248,8 +248,12 @@ def test_reconstruct_remainders_and_alignments_agree_bitwise(gc, n, dtype):
     (1, 6, 16, 16, 4, 2, 4, "bf16", "delta", False),    # one tile of 256 tokens, exactly
     (2, 6, 37, 29, 5, 5, 4, "bf16", "delta", True),     # ragged, two rounds of anchors, a channel group of 1
     (3, 12, 24, 40, 3, 9, 1, "f32", "copy", False),     # three rounds
-    (86, 6, 36, 32, 4, 2, 4, "bf16", "delta", False),   # 1,032 units with a last tile of 128 tokens: staged
-    (85, 6, 36, 32, 4, 3, 4, "f32", "copy", True),      # 1,020 units: one token per thread
+    (43, 6, 36, 32, 4, 2, 4, "bf16", "delta", False),   # 516 units with a last tile of 128 tokens: staged
+    (42, 6, 36, 32, 4, 3, 4, "f32", "copy", True),      # 504 units: one token per thread
+    (28, 12, 48, 48, 4, 3, 4, "bf16", "delta", True),   # 1,008 units of larger assets: one token per thread
+    (29, 12, 48, 48, 4, 4, 1, "f32", "delta", False),   # 1,044: staged
+    (86, 6, 36, 32, 4, 2, 4, "bf16", "copy", True),
+    (85, 6, 36, 32, 4, 3, 4, "f32", "copy", True),
     (33, 6, 37, 29, 4, 3, 4, "bf16", "copy", True),     # 396 units, unaligned rows: one CTA per tile
     (32, 6, 37, 29, 4, 2, 1, "f32", "delta", False),    # 384 units
 ])
