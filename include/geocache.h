@@ -452,8 +452,9 @@ int geocache_device_status(void* stream);
 /* --------------------------------------------------------------------------
  * geocache_debug_set_wait -- test hook of the failure handling (the paper has
  * no counterpart; not needed in normal use).  The staged transport kernel
- * (large steps in MASK mode with H*W % 8 == 0 and 16-byte aligned buffers; of any
- * size while drop_first_copy is pending) waits for its shared-memory copies
+ * (large steps in MASK mode, and in TABLE and GEOMETRY mode with one anchor, with
+ * H*W % 8 == 0 and 16-byte aligned buffers; MASK steps of any size while
+ * drop_first_copy is pending) waits for its shared-memory copies
  * with a time limit instead of spinning forever.
  *   limit_ns         limit of those waits for later calls (0 = the default, 2 s).
  *   drop_first_copy  nonzero: the next call that runs the staged kernel arms

@@ -1251,7 +1251,8 @@ __device__ __forceinline__ uint32_t quad_masks(const uint8_t* row, int cnt, bool
     return m;
 }
 
-// Large MASK steps: a persistent kernel whose CTAs loop over work units
+// Large MASK steps, and large TABLE and GEOMETRY steps with one anchor (see
+// launch_tiles): a persistent kernel whose CTAs loop over work units
 // (asset b, view v, tile of kTileTokens tokens, group of 4 channels).
 //  * Streaming: one thread arms the unit's mbarrier and issues TMA bulk
 //    copies (cp.async.bulk) of the unit's rows of x0 (the anchor's fresh x0,
@@ -1259,11 +1260,11 @@ __device__ __forceinline__ uint32_t quad_masks(const uint8_t* row, int cnt, bool
 //    ahead, so the next unit's rows are in flight while the current unit's
 //    increments are formed.
 //  * Increments (views outside the anchor set): the (token, anchor) pairs
-//    with a kept tap are compacted into a work list (block prefix sum, token
-//    order) and processed one per thread, so the dependent loads of many
-//    tokens overlap:  keep masks -> target position -> projection and
-//    weights -> gathers of the anchor increments x0_new - x0(t-1) at the kept
-//    taps.  Per-anchor sums are combined in anchor order (Eq. 1 with the
+//    with a kept tap (MASK; in the other modes every candidate pair) are
+//    compacted into a work list (block prefix sum, token order) and processed one
+//    per thread, so the dependent loads of many tokens overlap (MASK: keep masks
+//    -> target position -> projection and weights -> gathers of the anchor
+//    increments x0_new - x0(t-1) at the kept taps).  Per-anchor sums are combined in anchor order (Eq. 1 with the
 //    multi-anchor aggregation of Sec. 3.2: the mean over covering anchors; a
 //    token without a kept tap keeps x0(t-1)).
 //  * Every token is stored (x0(t)) and reconstructed (x_{t-1}) from the
@@ -1444,7 +1445,7 @@ __device__ __forceinline__ UnitCoord unit_coord(long long u, int n_tiles, int n_
 
 // Increments of the tile's covered tokens (views outside the anchor set),
 // left in sh.acc / sh.n for the tile's tokens.
-template <int K, bool VEC>
+template <int K, int MODE, bool VEC>
 __device__ __forceinline__ void tile_increments(const TransportArgs& args, FusedShared& sh, int b, int v, int tile0,
                                                 int cg, int cn) {
     const int HW = args.H * args.W;
@@ -1454,6 +1455,13 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     const int N = args.N, a = args.a;
     const size_t plane = (size_t)HW;
     const size_t tv0 = ((size_t)b * N + v) * plane;
+    float tau2 = 0.0f;
+    uint32_t fg = 0;  // GEOMETRY: validity bytes of the thread's tokens
+    if (MODE == GEOCACHE_CORR_GEOMETRY) {
+        const float tu = __ldg(args.tau + b);
+        tau2 = __fmul_rn(tu, tu);
+        if (cnt > 0) fg = quad_masks(args.valid + tv0 + p0, cnt, VEC);
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         *reinterpret_cast<float4*>(sh.acc[4 * t + i]) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1461,12 +1469,17 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     }
     for (int ac = 0; ac < a; ac += kChunk) {
         const int na = a - ac < kChunk ? a - ac : kChunk;
-        for (int i = t; i < na * 16; i += kThreads)
-            reinterpret_cast<float*>(sh.cam)[i] = __ldg(
-                reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (i >> 4)]) + (i & 15));
+        if (MODE != GEOCACHE_CORR_TABLE)
+            for (int i = t; i < na * 16; i += kThreads)
+                reinterpret_cast<float*>(sh.cam)[i] = __ldg(
+                    reinterpret_cast<const float*>(args.cams + (size_t)b * N + args.anchors[ac + (i >> 4)]) + (i & 15));
         // (token, anchor) work items of this anchor chunk
         uint32_t m4[4] = {0, 0, 0, 0};  // per own token: 4 bits per anchor of the chunk
-        if (cnt > 0) {
+        if (cnt > 0 && MODE != GEOCACHE_CORR_MASK) {  // every anchor is a candidate of a (foreground) token
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (MODE == GEOCACHE_CORR_TABLE ? i < cnt : ((fg >> (8 * i)) & 0xffu) != 0) m4[i] = (1u << (4 * na)) - 1u;
+        } else if (cnt > 0) {
             const uint8_t* krow = args.keep + ((size_t)b * N + v) * N * plane + p0;
             uint32_t q[kChunk];
 #pragma unroll
@@ -1502,7 +1515,7 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
                 const int s_loc = (int)((it >> 10) & 63u);
                 const int m = (int)((it >> 16) & 15u);
                 Taps tp;
-                item_taps<K, GEOCACHE_CORR_MASK>(args, sh.cam[s_loc], b, v, ac + s_loc, tile0 + lp, m, tv0, plane, 0.0f, tp);
+                item_taps<K, MODE>(args, sh.cam[s_loc], b, v, ac + s_loc, tile0 + lp, m, tv0, plane, tau2, tp);
                 if (tp.kept) {
                     item_increment<K>(args, tp, b, ac + s_loc, cg, cn, plane, g);
                     s_mine = s_loc;
@@ -1526,7 +1539,7 @@ __device__ __forceinline__ void tile_increments(const TransportArgs& args, Fused
     }
 }
 
-template <typename T, int K>
+template <typename T, int K, int MODE>
 __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const TransportArgs args, int n_tiles, int n_cg,
                                                                    long long n_units) {
     __shared__ FusedShared sh;
@@ -1582,7 +1595,7 @@ __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const Transpo
         const int cnt = p0 < HW ? (HW - p0 < 4 ? HW - p0 : 4) : 0;
         const int cn = C - c.cg < 4 ? C - c.cg : 4;
         const int slot = args.slot_of[c.v];
-        if (slot < 0) tile_increments<K, true>(args, sh, c.b, c.v, tile0, c.cg, cn);
+        if (slot < 0) tile_increments<K, MODE, true>(args, sh, c.b, c.v, tile0, c.cg, cn);
 
         const bool ok = mbar_wait_bounded(&sh.bar[st], parity[st], args.wait_limit_ns);
         if (__syncthreads_or(!ok)) {  // the whole CTA gives up together
@@ -1646,7 +1659,7 @@ __global__ void __launch_bounds__(kThreads) transport_fused_kernel(const Transpo
 // General path (sizes the bulk copies cannot serve: H*W not a multiple of 8
 // or buffers not 16-byte aligned): one CTA per unit, registers instead of
 // the shared-memory ring.
-template <typename T, int K, bool VEC>
+template <typename T, int K, int MODE, bool VEC>
 __global__ void __launch_bounds__(kThreads) transport_simple_kernel(const TransportArgs args, int n_tiles, int n_cg) {
     __shared__ FusedShared sh;
     const int t = threadIdx.x;
@@ -1678,7 +1691,7 @@ __global__ void __launch_bounds__(kThreads) transport_simple_kernel(const Transp
             if (recon) xt[cc] = Lat4<T>::load_raw(xt_p, view_base + (size_t)(c.cg + cc) * plane, cnt, VEC);
         }
     }
-    if (slot < 0) tile_increments<K, VEC>(args, sh, c.b, c.v, tile0, c.cg, cn);
+    if (slot < 0) tile_increments<K, MODE, VEC>(args, sh, c.b, c.v, tile0, c.cg, cn);
     if (cnt <= 0) return;
     if (slot < 0) {
 #pragma unroll
@@ -1740,7 +1753,7 @@ __device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_pt
     return (int)(x < 0 ? 0 : (x < cap ? x : cap));
 }
 
-// TABLE and GEOMETRY steps, and MASK and SPARSE steps of few units: one CTA per 256 tokens
+// Most TABLE and GEOMETRY steps, and MASK and SPARSE steps of few units: one CTA per 256 tokens
 // of a view and group of 4 channels, one token per thread, any alignment.
 // The two kernels above take a tile of 1024 tokens per CTA, whose work items
 // (token, anchor; up to 4 per token and round of anchors) go 256 at a time
@@ -1752,7 +1765,7 @@ __device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_pt
 // order (the same additions).  8 assets x 6 views of 96 x 96 x 4 bf16, 3 anchors,
 // against those kernels: masks 19.7 -> 12.0 us, tables (every token an item)
 // 50.4 -> 19.1, geometry 48.8 -> 17.9; 64 assets: tables 215 -> 144, geometry
-// 199 -> 137, so those take it at every size.
+// 199 -> 137.
 constexpr int kTokenAnchors = 4;  // anchors per round
 // resident CTAs per SM: 3 (80 registers, a few spilled) or 2, whichever was
 // faster: 8 assets, masks 12.0 / 12.2, geometry 17.9 / 17.9 (64 assets 137 / 155),
@@ -2715,8 +2728,27 @@ static cudaError_t launch_token(const TransportArgs& t, cudaStream_t s) {
     return launch_pdl(transport_token_kernel<T, K, MODE>, grid, kThreads, 0, s, t, make_fastdiv((uint32_t)n_cg));
 }
 
+// TABLE and GEOMETRY steps of at least this many units with one anchor (for
+// GEOMETRY on unaligned rows and f32 latents, two) keep the kernels with a tile of
+// 1024 tokens per CTA: the steps are then bound by their streams, which those
+// move in 16-byte words, and one item per token leaves no chain to shorten.
+// Token kernel and these (us; 6 views of 128 x 128, bf16): 1 anchor, 6,144 units of
+// C = 4: geometry 247 and 225, tables 226 and 198; of C = 16: 234 and 165, 217 and 171;
+// 1,056 units of C = 4: 34 and 41, 35 and 36; 2 anchors, 6,144 units of C = 4: 263 and 314, 281
+// and 289 (of C = 16: 252 and 223, 267 and 251, but 12 views of 64 x 64: 1.1 to 1.4
+// times faster by token).  With aligned rows, tables of single taps read a word per
+// item and are faster by token at every size (3,072 units of C = 4: 72 and 88), those
+// of f32 latents as fast.
+constexpr long long kTileUnitsItems = 1280;
 template <typename T, int K>
-static cudaError_t launch_mask(const TransportArgs& t, cudaStream_t s) {
+static bool items_by_tile(const TransportArgs& t, bool staged, long long n_units) {
+    if (n_units < kTileUnitsItems) return false;
+    if (t.mode == GEOCACHE_CORR_TABLE) return t.a == 1 && !(staged && (K == 1 || sizeof(T) == 4));
+    return t.a == 1 || (t.a == 2 && !staged && sizeof(T) == 4);
+}
+
+template <typename T, int K, int MODE>
+static cudaError_t launch_tiles(const TransportArgs& t, cudaStream_t s) {
     const int HW = t.H * t.W;
     const uintptr_t al = (uintptr_t)t.x0_new | (uintptr_t)t.x0_prev | (uintptr_t)t.x0_out | (uintptr_t)t.x_t |
                          (uintptr_t)t.x_next | (uintptr_t)t.pred_out | (uintptr_t)t.keep | (uintptr_t)t.valid;
@@ -2725,16 +2757,20 @@ static cudaError_t launch_mask(const TransportArgs& t, cudaStream_t s) {
     const int n_cg = (t.C + 3) / 4;
     const long long n_units = (long long)t.B * t.N * n_tiles * n_cg;
     const bool staged = vec && HW % 8 == 0;
-    // (a pending request of the test hook is for the staged kernel)
-    if (n_units <= mask_token_units(t, staged) && !(staged && g_drop_first_copy.load()))
-        return launch_token<T, K, GEOCACHE_CORR_MASK>(t, s);
+    if (MODE == GEOCACHE_CORR_MASK) {
+        // (a pending request of the test hook is for the staged kernel)
+        if (n_units <= mask_token_units(t, staged) && !(staged && g_drop_first_copy.load()))
+            return launch_token<T, K, MODE>(t, s);
+    } else if (!items_by_tile<T, K>(t, staged, n_units)) {
+        return launch_token<T, K, MODE>(t, s);
+    }
     // TMA bulk rows need 16-byte aligned starts and sizes: HW % 8 == 0 covers bf16 rows
     if (staged) {
         TransportArgs ta = t;
         ta.wait_limit_ns = g_wait_limit_ns.load();
         ta.drop_first_copy = g_drop_first_copy.exchange(0);
         const size_t dyn = kStages * 4 * kTileTokens * (sizeof(float) + sizeof(T));
-        auto kern = transport_fused_kernel<T, K>;
+        auto kern = transport_fused_kernel<T, K, MODE>;
         static int grid = 0;  // per instantiation and process (one device per process)
         if (!grid) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -2748,9 +2784,9 @@ static cudaError_t launch_mask(const TransportArgs& t, cudaStream_t s) {
     }
     if (n_units > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (vec)
-        transport_simple_kernel<T, K, true><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
+        transport_simple_kernel<T, K, MODE, true><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
     else
-        transport_simple_kernel<T, K, false><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
+        transport_simple_kernel<T, K, MODE, false><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
     return cudaGetLastError();
 }
 
@@ -2758,9 +2794,9 @@ template <typename T, int K>
 static cudaError_t launch_transport_t(const TransportArgs& t, cudaStream_t s) {
     switch (t.mode) {
         case GEOCACHE_CORR_SPARSE: return launch_sparse<T, K>(t, s);
-        case GEOCACHE_CORR_MASK: return launch_mask<T, K>(t, s);
-        case GEOCACHE_CORR_TABLE: return launch_token<T, K, GEOCACHE_CORR_TABLE>(t, s);
-        default: return launch_token<T, K, GEOCACHE_CORR_GEOMETRY>(t, s);
+        case GEOCACHE_CORR_MASK: return launch_tiles<T, K, GEOCACHE_CORR_MASK>(t, s);
+        case GEOCACHE_CORR_TABLE: return launch_tiles<T, K, GEOCACHE_CORR_TABLE>(t, s);
+        default: return launch_tiles<T, K, GEOCACHE_CORR_GEOMETRY>(t, s);
     }
 }
 

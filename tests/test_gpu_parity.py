@@ -256,6 +256,11 @@ def test_reconstruct_remainders_and_alignments_agree_bitwise(gc, n, dtype):
     (85, 6, 36, 32, 4, 3, 4, "f32", "copy", True),
     (33, 6, 37, 29, 4, 3, 4, "bf16", "copy", True),     # 396 units, unaligned rows: one CTA per tile
     (32, 6, 37, 29, 4, 2, 1, "f32", "delta", False),    # 384 units
+    (107, 6, 36, 32, 4, 1, 4, "bf16", "delta", False),  # 1,284 units, one anchor: tables and geometry by tile as well
+    (106, 6, 36, 32, 4, 1, 4, "f32", "copy", True),     # 1,272: by token
+    (54, 6, 36, 32, 7, 1, 1, "f32", "delta", True),     # 1,296, single taps: tables by token, geometry by tile
+    (107, 6, 37, 29, 4, 1, 4, "bf16", "copy", True),    # unaligned rows
+    (107, 6, 37, 29, 3, 2, 1, "f32", "delta", False),   # two anchors: geometry by tile
 ])
 def test_mode_kernels_agree_bitwise(gc, B, N, H, W, C, a, K, dtype, update, in_place):
     # every kernel that the MASK, TABLE and GEOMETRY steps choose between, against the sparse step
