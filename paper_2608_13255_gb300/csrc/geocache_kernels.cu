@@ -626,18 +626,27 @@ static void launch_build_corr_rep(const geocache_corr& c, int32_t* cnt, cudaStre
             c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx, c.w, c.keep, cnt, 1);
 }
 
-// Tiles from which the depth test pays for its two extra launches and its
-// fewer, larger CTAs (masks of 6 or 12 views at 128 x 128, old and new: 384
-// tiles 18.3 and 20.6 us, 768 tiles 27.7 and 25.3, 768 (12 views) 59.6 and 49.1,
-// 6,144 tiles 142 and 104; 600 tiles of 61 x 97: 17.2 and 17.4).
-constexpr long long kDepthTestTiles = 700;
+// Whether a build without tables tests depths first: where its fewer, larger CTAs
+// and two extra launches pay.  That takes tiles that are mostly full, or many views
+// to project into, and more tiles for single taps, which have less to skip, and for
+// masks whose rows are not 16-byte aligned, which are cleared in pieces.  tau,
+// masks and offsets without and with it, us: 6 views of 128 x 128: 384 tiles 26.4
+// and 28.6, 672 36.1 and 32.8, 5,952 175 and 121; of 64 x 64: 696 tiles 34.0 and 37.6,
+// 1,008 41.9 and 40.9; K = 1: 128 x 128 960 tiles 31.4 and 32.2, 1,440 39.7 and 39.0; 75 x
+// 53: 1,392 tiles 58.9 and 61.7, 1,992 82.0 and 81.4, K = 1 3,000 83.3 and 88.2, 6,000 156
+// and 158; 16 x 16: 6 views 6,000 tiles 95.7 and 117, 24 views 696 tiles 50.3 and 45.6.
+static bool depth_test_pays(const geocache_corr& c, long long tiles) {
+    const int HW = c.H * c.W;
+    if (HW < GEOCACHE_TILE_TOKENS && !(c.N >= 24 && c.K == 4)) return false;
+    return tiles >= (HW % 16 == 0 ? 700 : 1700) * (c.K == 4 ? 1 : 2);
+}
 
 cudaError_t launch_build_corr(const geocache_corr& c, cudaStream_t s) {
     const int HW = c.H * c.W, T = tiles_per_view(c.H, c.W);
     const long long tiles = (long long)T * c.N * c.B;
     const long long nb = (long long)depth_blocks(c.H) * depth_blocks(c.W);
     // the depths of a view fit its diagonal row (with 3 bytes to align them)
-    if (!c.idx && c.keep && tiles >= kDepthTestTiles && 4 * nb + 3 <= HW) {
+    if (!c.idx && c.keep && depth_test_pays(c, tiles) && 4 * nb + 3 <= HW) {
         const long long strips = (long long)((depth_blocks(c.W) + 3) / 4) * depth_blocks(c.H);
         source_depth_kernel<<<dim3((unsigned)((strips + 7) / 8), c.N, c.B), 256, 0, s>>>(c.pos, c.valid, c.cams, c.tau, c.N,
                                                                                    c.H, c.W, c.keep);

@@ -88,19 +88,25 @@ def test_tables_bit_exact_k1(gc, workloads, name):
 
 
 @pytest.mark.parametrize("H,W,B,K,scene", [(24, 21, 320, 4, "plain"), (24, 21, 320, 1, "plain"), (37, 29, 160, 4, "far"),
-                                           (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd"),
+                                           (40, 32, 160, 4, "scaled"), (16, 16, 320, 4, "odd"), (32, 32, 120, 4, "odd"),
                                            (37, 29, 1900, 4, "plain"),  # 136,800 counts: two rounds of the scan
-                                           (63, 65, 30, 4, "plain"), (63, 65, 30, 1, "offset"),
-                                           (126, 130, 8, 4, "plain"), (40, 32, 160, 4, "offset"),
+                                           (37, 29, 290, 1, "plain"), (32, 32, 234, 1, "far"), (16, 16, 30, 4, "views"),
+                                           (63, 65, 72, 4, "plain"), (63, 65, 142, 1, "offset"),
+                                           (126, 130, 18, 4, "plain"), (40, 32, 160, 4, "offset"),
                                            (40, 32, 160, 4, "minute"), (40, 32, 160, 4, "faint")])
 def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
-    # builds of at least 700 tiles test a source depth before the taps, and fill their records with a warp per tile
-    # from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
+    # builds of many tiles (of mostly full ones, or many views) test a source depth before the taps, and fill their
+    # records with a warp per tile from 8,192 tiles of pairs: masks, offsets and records equal those of each asset built alone (the small build
     # that the oracle checks).  far: an asset 3,000 units from the origin (the depths' rounding); scaled: cameras with
     # rows of other lengths than 1; faint and minute: rows, and positions, whose squares underflow; odd: infinite, huge
     # and NaN positions, and an empty asset; offset: masks 1 byte off their alignment (rows of 4,095 and 16,380 tokens
     # begin anywhere in a 16-byte word: the diagonal's last bytes)
     w = synth.make_workload("batch128", B=6, H=H, W=W)
+    if scene == "views":  # 24 of them, of tiles a quarter full
+        cams = np.stack([synth.look_at_camera(15.0 * i, 20.0 * (i % 3 - 1), H, W) for i in range(24)]).astype(np.float32)
+        pos, valid = synth.render_asset(synth.unit_sphere(), cams, H, W)
+        tile = lambda x: np.tile(x[None], (6,) + (1,) * x.ndim)
+        w = synth.Workload(**{**w.__dict__, "N": 24, "cams": tile(cams), "pos": tile(pos), "valid": tile(valid)})
     w.pos, w.cams = w.pos.copy(), w.cams.copy()
     R, t = w.cams[..., :9].reshape(6, w.N, 3, 3), w.cams[..., 9:12]
     if scene == "far":
