@@ -381,6 +381,7 @@ def measure_raster(dev, B, N_layout, H, W, reps=10, cpu_assets=2):
         gc.raster_posmaps(verts, faces, f_off, d_cams, H, W, zbuf, pos, valid)
     e1.record()
     torch.cuda.synchronize()
+    launches = gc.last_launches()
     gc.device_status()
     us = e0.elapsed_time(e1) * 1e3 / reps
     pixels, face_views = B * N * H * W, N * int(faces.shape[0])
@@ -390,7 +391,7 @@ def measure_raster(dev, B, N_layout, H, W, reps=10, cpu_assets=2):
     cpu_s = time.perf_counter() - t0
     return {"what": "%d meshes x %d views at %dx%d, 81920 faces each" % (B, N, H, W),
             "us_per_batch": us, "pixels_per_s": pixels / us * 1e6, "face_views_per_s": face_views / us * 1e6,
-            "covered_frac": float(valid.float().mean()), "launches_per_call": 2,
+            "covered_frac": float(valid.float().mean()), "launches_per_call": launches,
             "cpu_oracle": {"pixels_per_s": cpu_assets * N * H * W / cpu_s, "cores": 1,
                            "sample": "%d of the meshes, all views" % cpu_assets}}
 
@@ -535,16 +536,8 @@ class Trajectory:
         events: list receiving (start, end, 1) CUDA events around each cached step."""
         import torch
         gc, w = self.gc, self.w
-        launches = 0
         gc.build_corr(self.corr)
-        launches += 1 + (1 if (self.corr.idx is not None or self.corr.keep is not None) else 0)
-        tiles = w.B * w.N * gc.tiles_per_view(w.H, w.W)
-        if self.corr.idx is None and self.corr.keep is not None and tiles >= 700:
-            launches += 2  # large builds: the source depths before the masks, their clearing after
-        if self.corr.c.mode == gc.CORR_SPARSE:
-            launches += 2  # the tile offsets' scan, the records
-            if self.corr.c.src_ptr:
-                launches += 3  # the source index: counts, their scan, the scatter
+        launches = gc.last_launches()
         cache = None
         for t in range(w.S):
             timed = events is not None and t in self.anchor_x0
@@ -565,14 +558,11 @@ class Trajectory:
         anchors, full = gc.rotate_anchors(w.N, w.a, t, w.S, self.sched)
         if full:
             gc.reconstruct(self.x, self.full_x0[t], self.x, self.recon[t])
-            return self.full_x0[t], 1
+            return self.full_x0[t], gc.last_launches()
         out = self.bufs[0] if cache is not self.bufs[0] else self.bufs[1]
         gc.transport_step(self.corr, anchors, w.C, self.anchor_x0[t], cache, out, self.x, self.x, self.recon[t],
                           workspace=self.workspace)
-        units = w.B * w.N * gc.tiles_per_view(w.H, w.W) * -(-w.C // 4)
-        if self.corr.c.mode == gc.CORR_SPARSE and units <= 384:
-            return out, 1  # small steps that are not in place: one launch
-        return out, gc.transport_launches(w.a, w.N, self.corr.c.mode, in_place=False)
+        return out, gc.last_launches()
 
     def capture(self):
         """Capture the correspondence build and every sampler step in CUDA

@@ -506,6 +506,12 @@ int geocache_transport_step_noalloc(const geocache_corr* corr, const int32_t* an
  * none).  The pointer stays valid until the thread's next library call. */
 const char* geocache_last_error(void);
 
+/* Kernels that this thread's last enqueueing call (the entry points that take a
+ * stream, but for geocache_device_status) put on its stream; which kernels a call
+ * takes depends on its sizes, alignments and workspace.  0 for a call that was
+ * refused.  Host only. */
+int geocache_last_launches(void);
+
 /* GEOCACHE_ABI_VERSION of the loaded library. */
 int geocache_abi_version(void);
 

@@ -15,6 +15,7 @@
 namespace {
 
 thread_local std::string g_last_error;
+thread_local int g_launches = 0;  // kernels of the thread's last enqueueing call
 
 int fail(int status, const char* fmt, ...) {
     char buf[512];
@@ -176,10 +177,15 @@ int geocache::set_error(int status, const char* fmt, ...) {
     vsnprintf(buf, sizeof buf, fmt, ap);
     va_end(ap);
     g_last_error = buf;
+    g_launches = 0;
     return status;
 }
 
+void geocache::note_launches(int n) { g_launches += n; }
+
 extern "C" {
+
+int geocache_last_launches(void) { return g_launches; }
 
 int geocache_abi_version(void) { return GEOCACHE_ABI_VERSION; }
 
@@ -213,6 +219,7 @@ int geocache_debug_set_wait(uint64_t limit_ns, int drop_first_copy) {
 }
 
 int geocache_build_corr(geocache_corr* c, void* stream) {
+    g_launches = 0;
     const int st = check_build(c);
     if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
@@ -230,6 +237,7 @@ int geocache_build_corr(geocache_corr* c, void* stream) {
 }
 
 int geocache_fill_records(geocache_corr* c, void* stream) {
+    g_launches = 0;
     const int st = check_build(c);
     if (st) return st;
     if (!c->keep || !c->tile_ptr || !c->records)
@@ -238,6 +246,7 @@ int geocache_fill_records(geocache_corr* c, void* stream) {
 }
 
 int geocache_corr_record_count(geocache_corr* c, int64_t* count, void* stream) {
+    g_launches = 0;
     if (!c || !count) return fail(GEOCACHE_EINVAL, "corr and count are required");
     if (!c->keep || !c->tile_ptr) return fail(GEOCACHE_EINVAL, "counting records needs keep and tile_ptr");
     geocache_corr d = *c;
@@ -273,6 +282,7 @@ int geocache_transport_step_update(const geocache_corr* c, geocache_update updat
                                    const void* x_t, void* x_next, geocache_dtype lat_dtype,
                                    const geocache_recon* recon, float* workspace, int64_t workspace_floats,
                                    void* stream) {
+    g_launches = 0;
     if (!c) return fail(GEOCACHE_EINVAL, "corr is NULL");
     if (update != GEOCACHE_UPDATE_DELTA && update != GEOCACHE_UPDATE_COPY)
         return fail(GEOCACHE_EINVAL, "unknown update rule %d", (int)update);
@@ -372,6 +382,7 @@ int geocache_transport_step_update(const geocache_corr* c, geocache_update updat
 }
 
 int geocache_permute_records(const geocache_corr* c, const int32_t* perm, geocache_tap_record* out, void* stream) {
+    g_launches = 0;
     if (!c || !perm || !out) return fail(GEOCACHE_EINVAL, "corr, perm and out are required");
     if (!c->records || c->max_records < 0) return fail(GEOCACHE_EINVAL, "corr has no sparse records");
     if (((uintptr_t)out | (uintptr_t)c->records) & 15) return fail(GEOCACHE_EINVAL, "records must be 16-byte aligned");
@@ -386,6 +397,7 @@ int geocache_permute_records(const geocache_corr* c, const int32_t* perm, geocac
 static int raster_entry(const char* fn, const float* verts, int64_t n_verts, const int32_t* faces, int64_t n_faces,
                         const int64_t* face_off, int B, const geocache_camera* cams, int N, int H, int W, int ss,
                         uint64_t* zbuf, float* pos, uint8_t* valid, void* stream) {
+    g_launches = 0;
     if (B < 1 || B > 65535 || N < 1 || N > GEOCACHE_MAX_VIEWS || H < 1 || W < 1 || H > 16384 || W > 16384)
         return fail(GEOCACHE_ESHAPE, "%s: B=%d, N=%d, H=%d, W=%d out of range", fn, B, N, H, W);
     if (ss < 1 || ss > 16 || (int64_t)H * ss > 16384 || (int64_t)W * ss > 16384)
@@ -430,6 +442,7 @@ int geocache_raster_posmaps_supersampled(const float* verts, int64_t n_verts, co
 
 int geocache_pool_posmaps(const float* pos_hi, const uint8_t* valid_hi, int64_t n_maps, int H, int W, int s, float* pos,
                           uint8_t* valid, void* stream) {
+    g_launches = 0;
     if (n_maps < 0 || H < 1 || W < 1 || H > 16384 || W > 16384)
         return fail(GEOCACHE_ESHAPE, "geocache_pool_posmaps: n_maps=%lld, H=%d, W=%d out of range", (long long)n_maps, H, W);
     if (s < 1 || s > 16 || (int64_t)H * s > 16384 || (int64_t)W * s > 16384)
@@ -447,6 +460,7 @@ int geocache_pool_posmaps(const float* pos_hi, const uint8_t* valid_hi, int64_t 
 
 int geocache_reconstruct(const void* x_t, const float* x0, void* x_next, geocache_dtype lat_dtype, int64_t n,
                          const geocache_recon* recon, float* x0_store, void* stream) {
+    g_launches = 0;
     if (n < 0) return fail(GEOCACHE_ESHAPE, "n=%lld is negative", (long long)n);
     if (!recon) return fail(GEOCACHE_EINVAL, "recon is NULL");
     if (lat_dtype != GEOCACHE_F32 && lat_dtype != GEOCACHE_BF16)
@@ -475,6 +489,7 @@ int geocache_reconstruct(const void* x_t, const float* x0, void* x_next, geocach
 static int copy_rows_entry(const void* src, void* dst, int64_t row_bytes, int B, int N, const int32_t* anchors, int a,
                            bool pack, void* stream) {
     const char* fn = pack ? "geocache_pack_anchors" : "geocache_unpack_anchors";
+    g_launches = 0;
     if (B < 0 || B > 65535) return fail(GEOCACHE_ESHAPE, "%s: B=%d out of range [0, 65535]", fn, B);
     if (N < 1 || N > GEOCACHE_MAX_VIEWS) return fail(GEOCACHE_ESHAPE, "%s: N=%d out of range [1, %d]", fn, N, GEOCACHE_MAX_VIEWS);
     if (row_bytes < 0) return fail(GEOCACHE_ESHAPE, "%s: row_bytes=%lld is negative", fn, (long long)row_bytes);

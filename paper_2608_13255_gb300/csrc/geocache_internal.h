@@ -99,6 +99,10 @@ cudaError_t launch_raster(const float* V, long long nv, const int32_t* F, long l
 cudaError_t launch_pool_posmaps(const float* pos_hi, const uint8_t* valid_hi, long long n_maps, int H, int W, int ss,
                                 float* pos, uint8_t* valid, cudaStream_t s);
 
+// Counts kernels that the calling thread's current library call enqueues
+// (geocache_last_launches).
+void note_launches(int n);
+
 // Launch with programmatic stream serialization: the kernel may become resident
 // while the one before it in the stream drains, and begins with pdl_wait, before
 // it touches memory.  It hides the launch behind the predecessor's tail (us a
@@ -116,6 +120,7 @@ cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, size_t d
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    note_launches(1);
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
 }
 

@@ -211,6 +211,7 @@ cudaError_t launch_tau(const float* pos, const uint8_t* valid, int B, int N, int
     cfg.numAttrs = 1;
     // quads: every view's texels start on a 4-texel boundary with 16-byte aligned positions
     const int quads = (H * W) % 4 == 0 && (uintptr_t)pos % 16 == 0 && (uintptr_t)valid % 4 == 0;
+    note_launches(1);
     return cudaLaunchKernelEx(&cfg, tau_kernel, pos, valid, N, H * W, tol_frac, quads, tau);
 }
 
@@ -618,6 +619,7 @@ static void launch_build_corr_rep(const geocache_corr& c, int32_t* cnt, cudaStre
     const int HW = c.H * c.W, gx = (HW + kBuildThreads * REP - 1) / (kBuildThreads * REP);
     const long long ctas = (long long)gx * c.N * c.B, want = (kBuildCtas + ctas - 1) / ctas;
     const int n_split = (int)(want < c.N ? want : c.N);
+    note_launches(1);
     if (REP == 1 && n_split > 1)
         build_corr_kernel<K, TABLES, 1, true><<<dim3(gx, c.N * n_split, c.B), kBuildThreads, 0, s>>>(
             c.pos, c.valid, c.cams, c.tau, c.N, c.H, c.W, c.idx, c.w, c.keep, cnt, n_split);
@@ -658,6 +660,7 @@ cudaError_t launch_build_corr(const geocache_corr& c, cudaStream_t s) {
                                                                              c.W, c.keep, c.tile_ptr);
         const int chunks = HW / 16 + 2;  // of a row that starts anywhere in a 16-byte word (clear_chunk)
         clear_diagonal_kernel<<<dim3((unsigned)((chunks + 255) / 256), c.N, c.B), 256, 0, s>>>(c.keep, c.N, HW);
+        note_launches(3);
         return cudaGetLastError();
     }
     int32_t* cnt = nullptr;
@@ -788,6 +791,7 @@ __global__ void __launch_bounds__(1024) exclusive_scan_kernel(int32_t* a, long l
 }
 
 static cudaError_t launch_scan(int32_t* a, long long n, cudaStream_t s) {
+    note_launches(1);
     if (n <= 1024LL * kScanPer) {  // one round of one CTA, whose barrier is cheaper than the cluster's
         exclusive_scan_kernel<1><<<1, 1024, 0, s>>>(a, n);
         return cudaGetLastError();
@@ -1043,6 +1047,7 @@ template <int K>
 static void launch_fill_records_k(const geocache_corr& c, cudaStream_t s) {
     const int T = tiles_per_view(c.H, c.W);
     const long long tiles = (long long)T * c.N * (c.N - 1);  // per asset
+    note_launches(1);
     if (tiles * c.B >= kFillWarpTiles)
         fill_records_kernel<K><<<dim3((unsigned)((tiles + kFillWarps - 1) / kFillWarps), c.B), 32 * kFillWarps, 0, s>>>(
             c.pos, c.cams, c.keep, c.tile_ptr, c.N, c.H, c.W, T, c.records, c.max_records);
@@ -1102,6 +1107,7 @@ cudaError_t launch_src_index(const geocache_corr& c, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const dim3 grid(T, c.N * c.N, c.B);
     int2* out = reinterpret_cast<int2*>(c.src_rec);
+    note_launches(2);  // the counts and the scatter
     if (c.K == 4)
         src_index_kernel<4, false><<<grid, 256, 0, s>>>(c.tile_ptr, c.records, c.max_records, c.N, c.W, T, c.src_ptr, out);
     else
@@ -2674,6 +2680,7 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
             phase_a = true;
         }
     }
+    if (phase_a) note_launches(1);
     // an in-place update streams the anchor views after the wait, except with
     // the plane (its phase A reads each anchor element before writing it)
     const int gy = (t.N - t.a) + (in_place && !by_plane ? t.a : 0);
@@ -2702,6 +2709,7 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
             else e = cudaLaunchKernelEx(&cfg, sparse_phase_b_kernel<T, false, true, 0>, t, sg);
         }
         if (e != cudaSuccess) return e;
+        note_launches(1);
     }
     return cudaGetLastError();
 }
@@ -2788,10 +2796,12 @@ static cudaError_t launch_tiles(const TransportArgs& t, cudaStream_t s) {
             if (!grid) return cudaErrorInvalidConfiguration;
         }
         const long long g = n_units < grid ? n_units : grid;
+        note_launches(1);
         kern<<<(unsigned)g, kThreads, dyn, s>>>(ta, n_tiles, n_cg, n_units);
         return cudaGetLastError();
     }
     if (n_units > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    note_launches(1);
     if (vec)
         transport_simple_kernel<T, K, MODE, true><<<(unsigned)n_units, kThreads, 0, s>>>(t, n_tiles, n_cg);
     else
@@ -2830,6 +2840,7 @@ __global__ void copy_anchor_rows_kernel(const TransportArgs args) {
 cudaError_t launch_copy_anchor_rows(const TransportArgs& t, cudaStream_t s) {
     const size_t per = (size_t)t.cn * t.H * t.W;
     dim3 grid((unsigned)((per + 255) / 256), t.a, t.B);
+    note_launches(1);
     copy_anchor_rows_kernel<<<grid, 256, 0, s>>>(t);
     return cudaGetLastError();
 }
@@ -2884,6 +2895,7 @@ cudaError_t launch_permute_records(const geocache_tap_record* src, const int32_t
                                    long long n, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const long long blocks = (n + 255) / 256;
+    note_launches(1);
     permute_records_kernel<<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(
         reinterpret_cast<const int4*>(src), perm, reinterpret_cast<int4*>(dst), n);
     return cudaGetLastError();
@@ -2900,6 +2912,7 @@ cudaError_t launch_copy_rows(const void* src, void* dst, long long row_bytes, in
     dim3 grid((unsigned)gx, a, B);
     const uint8_t* sp = static_cast<const uint8_t*>(src);
     uint8_t* dp = static_cast<uint8_t*>(dst);
+    note_launches(1);
     if (vb == 16)
         copy_rows_kernel<16><<<grid, 256, 0, s>>>(sp, dp, row_bytes, N, a, anc, pack);
     else if (vb == 4)
@@ -2976,6 +2989,7 @@ static cudaError_t launch_reconstruct_t(const void* x_t, const float* x0, void* 
     const int64_t blocks8 = (n + 2047) / 2048;
     if (f32s % 32 == 0 && lats % (8 * sizeof(T)) == 0 && blocks8 <= 0x7fffffffLL)
         return launch_pdl(reconstruct8_kernel<T>, dim3((unsigned)blocks8), 256, 0, s, xt, x0, xn, n, coef, pred_out, x0_store);
+    note_launches(1);
     if (al % 16 == 0)
         reconstruct_kernel<T, true><<<(unsigned)blocks, 256, 0, s>>>(xt, x0, xn, n, coef, pred_out, x0_store);
     else

@@ -643,11 +643,13 @@ cudaError_t launch_raster(const float* V, long long nv, const int32_t* F, long l
         const RasterSplit split = raster_split(nf, B, N, (long long)H * W * ss * ss);
         const long long per_cta = split.faces * (kRasterThreads / 32), gx = (nf + per_cta - 1) / per_cta;
         if (gx > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        note_launches(1);
         raster_faces_kernel<<<dim3((unsigned)gx, (unsigned)((N + split.views - 1) / split.views)), kRasterThreads, 0, s>>>(
             V, nv, F, nf, face_off, B, cams, N, split, H * ss, W * ss, (float)ss, zbuf);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
+    note_launches(1);
     if (ss == 1)
         raster_resolve_kernel<<<stride_grid(n_pix), kRasterThreads, 0, s>>>(zbuf, cams, N, H, W, n_pix, pos, valid);
     else {

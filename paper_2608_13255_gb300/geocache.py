@@ -74,7 +74,7 @@ EXPORTS = ("geocache_build_corr", "geocache_transport_step", "geocache_reconstru
            "geocache_transport_workspace", "geocache_transport_step_noalloc", "geocache_pack_anchors",
            "geocache_unpack_anchors", "geocache_transport_step_update", "geocache_permute_records",
            "geocache_raster_posmaps", "geocache_debug_set_wait", "geocache_raster_posmaps_supersampled",
-           "geocache_pool_posmaps", "geocache_fill_records",
+           "geocache_pool_posmaps", "geocache_fill_records", "geocache_last_launches",
            "geocache_last_error", "geocache_abi_version")
 
 
@@ -127,6 +127,8 @@ def load():
         L.geocache_last_error.restype = ctypes.c_char_p
         L.geocache_last_error.argtypes = []
         L.geocache_abi_version.argtypes = []
+        L.geocache_last_launches.argtypes = []
+        L.geocache_last_launches.restype = ctypes.c_int
         for name in EXPORTS[:7]:
             getattr(L, name).restype = ctypes.c_int
         L.geocache_abi_version.restype = ctypes.c_int
@@ -516,12 +518,17 @@ def rotate_anchors(N: int, a: int, step: int, S: int, sched: dict):
     return list(out), bool(full.value)
 
 
+def last_launches() -> int:
+    """Kernels that this thread's last enqueueing call put on its stream."""
+    return load().geocache_last_launches()
+
+
 def transport_launches(a: int, N: int, mode: int, in_place: bool = False) -> int:
-    """Kernels one geocache_transport_step enqueues for a large batch: sparse mode
-    runs the record-parallel apply (when some view is outside the anchor set)
-    and the streaming kernel (small steps that are not in place: one kernel);
-    the other modes one fused kernel, plus the anchor-row copy of an in-place
-    update."""
+    """The most kernels a geocache_transport_step of these arguments enqueues:
+    sparse mode runs phase A (when some view is outside the anchor set) and the
+    streaming kernel, the other modes one kernel, plus the anchor-row copy of an
+    in-place update.  A small sparse step takes one (last_launches() after the
+    call is exact)."""
     if mode == CORR_SPARSE:
         return 2 if a < N else 1
     return 1 + (1 if in_place else 0)

@@ -808,6 +808,28 @@ def test_sparse_paths_of_large_steps_agree_bitwise(gc, B, N, H, W, C, a, K, dtyp
     assert not torch.equal(ref[0], x0.view(torch.uint8))
 
 
+@pytest.mark.parametrize("B,mode,a,in_place,launches", [
+    (2, "sparse", 2, False, 1), (2, "sparse", 2, True, 2), (60, "sparse", 2, False, 2), (2, "sparse", 6, False, 1),
+    (2, "mask", 2, False, 1), (2, "mask", 2, True, 2), (60, "mask", 2, True, 2), (2, "geometry", 2, False, 1)])
+def test_launches_are_counted(gc, B, mode, a, in_place, launches):
+    w = synth.replicate_assets(synth.make_workload("batch128", B=2, H=64, W=64), B)
+    pos, valid, cams = (torch.from_numpy(x).cuda() for x in (w.pos, w.valid, w.cams))
+    c = gc.build_sparse_corr(pos, valid, cams, source_index=True)
+    assert gc.last_launches() == 1 + 3  # the records and their source index (the count came before)
+    gc.build_corr(c)
+    assert gc.last_launches() == (7 if B * w.N * 4 < 700 else 9)  # large builds: depths before, the diagonal after
+    c.c.mode = {"sparse": gc.CORR_SPARSE, "mask": gc.CORR_MASK, "geometry": gc.CORR_GEOMETRY}[mode]
+    anchors = list(range(a))
+    x0 = torch.zeros((B, w.N, w.C, w.H, w.W), device="cuda")
+    ws = torch.empty(max(4, c.workspace_floats(w.C)), device="cuda")
+    gc.transport_step(c, anchors, w.C, x0[:, :a].contiguous(), x0, x0 if in_place else torch.empty_like(x0), workspace=ws)
+    assert gc.last_launches() == launches <= gc.transport_launches(a, w.N, c.c.mode, in_place)
+    with pytest.raises(gc.GeocacheError):  # refused: nothing enqueued
+        gc.transport_step(c, [1, 1], w.C, x0[:, :2].contiguous(), x0, torch.empty_like(x0), workspace=ws)
+    assert gc.last_launches() == 0
+    gc.device_status()
+
+
 def test_wide_views_fall_back_to_the_record_parallel_apply(gc):
     # W + 1 > 1024 tokens: the staged span of a source tile would not fit, so a
     # step with a source index and a minimal workspace applies the records
