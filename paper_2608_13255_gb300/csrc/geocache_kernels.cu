@@ -194,9 +194,8 @@ __global__ void __launch_bounds__(256, kTauBlocks) tau_kernel(const float* __res
 
 cudaError_t launch_tau(const float* pos, const uint8_t* valid, int B, int N, int H, int W, float tol_frac,
                        float* tau, cudaStream_t s) {
-    // a cluster of 8 CTAs (the portable size) per asset: 1024 CTAs for 128
-    // assets, resident at once at 8 per SM (one CTA per view at 512 threads,
-    // 768 CTAs in 1.3 waves, took 16 us more per 128-asset build)
+    // a cluster of 8 CTAs (the portable size) per asset, 4 CTAs resident per SM
+    // (64 registers: the loads in flight)
     const int cs = 8;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(B * cs);
@@ -611,7 +610,7 @@ __global__ void __launch_bounds__(256) clear_diagonal_kernel(uint8_t* keep, int 
 // fewer, a CTA's views in sequence are the time of the kernel: one asset of 6
 // views at 64 x 64 (96 CTAs) 7.5 us, with its views split over 576 CTAs 4.3; 4
 // views at 96 x 96 (144) 5.4 and 4.0, 8 at 64 x 64 (128) 9.5 and 5.7.  From 384 CTAs (6 views at 128 x 128)
-// on the split gains nothing (8.6 and 8.3), beyond 608 it loses.
+// on the split gains nothing (8.6 and 8.3), beyond 608 (4 per SM) it loses.
 constexpr long long kBuildCtas = 608;
 
 template <int K, bool TABLES, int REP>
@@ -2197,7 +2196,7 @@ template <typename T>
 constexpr int kPhaseBBlocks = sizeof(T) == 2 ? 5 : 1;
 // The increment-plane kernels (wide latents): phase A at 4 resident CTAs per
 // SM (62 registers; at 5 or 6 its spills cost more than the residency
-// gains), phase B at 5 (46 registers, no spills: it loads its streamed rows
+// gains), phase B at 5 (45 registers for 4 taps of bf16: it loads its streamed rows
 // after the fold, so they are not held across the gathers; 4 or 6 resident
 // CTAs, or the rows prefetched into the L2 before the wait, were slower).
 constexpr int kPlaneABlocks = 4;

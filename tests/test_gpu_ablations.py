@@ -84,7 +84,7 @@ def _pair_counts(g, w):
 def test_shuffled_correspondence_parity(gc, workloads, name):
     w = workloads(name)
     if name == "batch128":
-        w = synth.make_workload("batch128", B=2)
+        w = synth.make_workload("batch128", B=5)  # 480 units: two launches
     g = DeviceGeometry(w, K=w.K, tables=False)
     tau = oracle.tau(w.pos, w.valid, w.tol_frac)
     idx, wt, _ = oracle.build_corr(w.pos, w.valid, w.cams, tau, K=w.K, with_band=False)

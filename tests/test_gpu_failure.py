@@ -76,19 +76,38 @@ def test_wait_that_runs_out_is_reported_and_the_context_stays_usable(gc, workloa
     assert_bf16_close(xn2.cpu().view(torch.int16).numpy().view(np.uint16), ref_xn, what="x_next after the timeout")
 
 
-def test_wait_limit_restored_by_default(gc, workloads):
-    # a short limit that every copy meets: no timeout is reported
-    w = workloads("hunyuan64")
+def test_waits_that_end_in_time_report_nothing(gc, workloads):
+    # the staged kernel (528 units: MASK steps of at most 512 take another), under a limit that every copy meets and
+    # after a timeout: complete, correct, no timeout reported
+    w = synth.replicate_assets(workloads("hunyuan64"), 22)
     g = DeviceGeometry(w, K=4, tables=False)
+    corr = g.corr_for("mask")
     anchors = [1, 4]
-    x0_prev, x0_new, _, _ = _inputs(w, anchors)
-    d_prev, d_new = torch.from_numpy(x0_prev).cuda(), torch.from_numpy(x0_new).cuda()
-    gc.debug_set_wait(100_000_000)  # 100 ms
-    try:
-        out = torch.empty_like(d_prev)
-        gc.transport_step(g.corr_for("mask"), anchors, w.C, d_new, d_prev, out)
+    x0_prev, x0_new, xt64, xt = _inputs(w, anchors)
+    p = synth.recon_params(w, 4)
+    r = gc.make_recon("ddim", a_t=p["a_t"], a_prev=p["a_prev"])
+    d_prev, d_new, d_xt = torch.from_numpy(x0_prev).cuda(), torch.from_numpy(x0_new).cuda(), xt.cuda()
+    tau = oracle.tau(w.pos, w.valid, w.tol_frac)
+    ref_x0, ref_xn, _ = oracle.transport_step(anchors, x0_new, x0_prev, K=4, geom=(w.pos, w.valid, w.cams, tau),
+                                              x_t=xt64, recon=recon_kw(p))
+
+    def step():
+        out, xn = torch.full_like(d_prev, float("nan")), torch.empty_like(d_xt)
+        gc.transport_step(corr, anchors, w.C, d_new, d_prev, out, d_xt, xn, r)
         torch.cuda.synchronize()
-        gc.device_status()
+        return out, xn
+
+    try:
+        gc.debug_set_wait(200_000, drop_first_copy=True)
+        assert torch.isnan(step()[0][0, 0]).any()  # unit 0 was dropped: this size runs the staged kernel
+        with pytest.raises(gc.GeocacheError) as ei:
+            gc.device_status()
+        assert ei.value.status == gc.ETIMEOUT
+        for limit_ns in (0, 100_000_000):
+            gc.debug_set_wait(limit_ns)
+            out, xn = step()
+            gc.device_status()
+            assert_f32_close(out.cpu().numpy(), ref_x0, what="x0")
+            assert_bf16_close(xn.cpu().view(torch.int16).numpy().view(np.uint16), ref_xn, what="x_next")
     finally:
         gc.debug_set_wait(0)
-    assert torch.isfinite(out).all()

@@ -83,25 +83,31 @@ def _geometry(gc, w, K=4, skew=0, records_frac=1.0):
     return corr, g, R, cap, (pos, valid, cams)
 
 
-@pytest.mark.parametrize("case", ["ragged_c5", "ragged_c18", "ragged_c18_src", "misaligned", "c3_k1"])
-def test_transport_writes_only_its_outputs(gc, case):
-    minimal_ws = False
+@pytest.mark.parametrize("case,B,a", [
+    ("ragged_c5", 2, 2), ("ragged_c5", 20, 2),    # one token per thread; beside it two launches, masks by tile
+    ("ragged_c18", 2, 2), ("ragged_c18", 9, 2), ("ragged_c18_src", 9, 2), ("ragged_c18_src", 2, 2),
+    ("misaligned", 1, 2), ("misaligned", 22, 2),
+    ("c3_k1", 1, 2), ("c3_k1", 110, 1),           # masks and geometry by tile from staged rows
+    ("aligned_c6", 22, 3)])
+def test_transport_writes_only_its_outputs(gc, case, B, a):
+    minimal_ws = case == "ragged_c18_src"  # the source-tile apply instead of the increment plane
     if case == "ragged_c5":  # 37 x 53 tokens: H*W = 1961, two tiles, a ragged quad; C = 5
         w, C, skew, K = synth.make_workload("batch128", B=2, H=37, W=53), 5, 0, 4
-    elif case == "ragged_c18":  # the same with C = 18: the increment plane, a partial last channel group
+    elif case in ("ragged_c18", "ragged_c18_src"):  # the same with C = 18: a partial last channel group
         w, C, skew, K = synth.make_workload("batch128", B=2, H=37, W=53), 18, 0, 4
-    elif case == "ragged_c18_src":  # C = 18 with the minimal workspace: the source-tile apply
-        w, C, skew, K = synth.make_workload("batch128", B=2, H=37, W=53), 18, 0, 4
-        minimal_ws = True
     elif case == "misaligned":  # 64 x 64 tokens, every buffer 4 bytes off a 16-byte boundary
         w, C, skew, K = synth.make_workload("hunyuan64"), 4, 4, 4
+    elif case == "aligned_c6":  # 64 x 64 tokens, 16-byte words
+        w, C, skew, K = synth.make_workload("batch128", B=2, H=64, W=64), 6, 0, 4
     else:
         w, C, skew, K = synth.make_workload("solids96", H=40, W=40), 3, 0, 1
-    w = synth.Workload(**{**w.__dict__, "C": C})
+    w = synth.replicate_assets(synth.Workload(**{**w.__dict__, "C": C}), B)
     corr, g, R, cap, _ = _geometry(gc, w, K=K, skew=skew)
     for k, v in g.items():
         v.check("build: " + k)
-    anchors = [0, 3]
+    anchors = [0, 3, 4][:a]
+    # sparse steps of few units take one launch without the workspace, the others two
+    two = B > 2
     x0_prev, x0_new, xt32 = step_inputs(w, 3, anchors)
     shp = (w.B, w.N, C, w.H, w.W)
     lat = torch.bfloat16 if w.dtype == "bf16" else torch.float32
@@ -126,7 +132,10 @@ def test_transport_writes_only_its_outputs(gc, case):
         d_xt = Guarded(shp, lat, skew, torch.from_numpy(xt32).to(lat))
         gc.transport_step(c2, anchors, C, d_new.t, d_prev.t, out.t, d_xt.t, xn.t, r,
                           workspace=ws.t if mode == "sparse" else None)
+        assert gc.last_launches() == (2 if mode == "sparse" and two else 1)
         gc.device_status()
+        if mode == "sparse":
+            assert bool((ws.t.view(torch.uint8) != SENTINEL).any()) == two
         for name, gb in (("x0_out", out), ("x_next", xn), ("pred", pred), ("workspace", ws), ("x0_prev", d_prev),
                          ("x0_new", d_new), ("x_t", d_xt)):
             gb.check("%s %s: %s" % (case, mode, name))
@@ -136,18 +145,21 @@ def test_transport_writes_only_its_outputs(gc, case):
             gc.transport_step(c2, anchors, C, d_new.t, d_prev.t, d_prev.t, d_xt.t, d_xt.t, r,
                               workspace=ws.t if mode == "sparse" else None)
             gc.device_status()
-            d_prev.check("%s %s in place: x0" % (case, mode))
-            d_xt.check("%s %s in place: x_t" % (case, mode))
+            for name, gb in (("x0", d_prev), ("x_t", d_xt), ("pred", pred), ("workspace", ws), ("x0_new", d_new)):
+                gb.check("%s %s in place: %s" % (case, mode, name))
+            if mode == "sparse":  # two launches at every size
+                assert gc.last_launches() == 2 and bool((ws.t.view(torch.uint8) != SENTINEL).any())
 
 
+@pytest.mark.parametrize("B", [2, 44])
 @pytest.mark.parametrize("frac,C", [(1.0, 4), (0.5, 4), (1.0, 16), (0.5, 16)])
-def test_record_buffer_at_and_beyond_capacity(gc, frac, C):
+def test_record_buffer_at_and_beyond_capacity(gc, frac, C, B):
     # records filled exactly to max_records, and an overflowing build (half
     # the capacity needed): nothing is written past the buffer, the overflow
     # is reported, and a step over the truncated form stays inside its outputs
-    # (C = 16: the increment-plane path)
+    # (2 assets: one launch; 44: the record-parallel apply, C = 16 the increment plane)
     w = synth.make_workload("batch128", B=2, H=37, W=53)
-    w = synth.Workload(**{**w.__dict__, "C": C})
+    w = synth.replicate_assets(synth.Workload(**{**w.__dict__, "C": C}), B)
     corr, g, R, cap, _ = _geometry(gc, w, K=4)
     if frac < 1.0:
         corr, g, R, cap, _ = _geometry(gc, w, K=4, records_frac=frac)
@@ -165,6 +177,8 @@ def test_record_buffer_at_and_beyond_capacity(gc, frac, C):
     ws = Guarded((corr.workspace_floats(w.C),), torch.float32)
     gc.transport_step(corr, [1, 4], w.C, torch.from_numpy(x0_new).cuda(), torch.from_numpy(x0_prev).cuda(), out.t,
                       workspace=ws.t)
+    assert gc.last_launches() == (1 if B == 2 else 2)
+    assert bool((ws.t.view(torch.uint8) != SENTINEL).any()) == (B > 2)
     gc.device_status()
     out.check("step over %d of %d records: x0_out" % (cap, R))
     ws.check("step over %d of %d records: workspace" % (cap, R))

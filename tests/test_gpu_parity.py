@@ -150,8 +150,9 @@ def test_large_builds_equal_small_ones(gc, H, W, B, K, scene):
 
 
 def _run_step(gc, w, g, anchors, params, pred=None, mode="sparse", inplace=False, xinplace=False,
-              seed_extra=0, C=None, minimal_ws=False):
-    """One cached step on the GPU and in the oracle from the same inputs."""
+              seed_extra=0, C=None, minimal_ws=False, launches=None):
+    """One cached step on the GPU and in the oracle from the same inputs
+    (launches: the kernels it must take)."""
     if C is not None and C != w.C:
         w = synth.Workload(**{**w.__dict__, "C": C})
     x0_prev, x0_new, xt32 = step_inputs(w, 3, anchors, seed_extra)
@@ -169,6 +170,7 @@ def _run_step(gc, w, g, anchors, params, pred=None, mode="sparse", inplace=False
                       pred_kind=pred, pred_out=d_pred)
     gc.transport_step(corr, anchors, w.C, d_new, d_prev, d_out, d_xt, d_xn, r,
                       workspace=g.workspace(w.C, minimal=minimal_ws))
+    assert launches is None or gc.last_launches() == launches
     torch.cuda.synchronize()
     gc.device_status()
     tau_ref = oracle.tau(w.pos, w.valid, w.tol_frac)
@@ -231,16 +233,27 @@ def test_corr_modes_agree_bitwise(gc, workloads, name, K):
 @pytest.mark.parametrize("n", [1, 7, 8, 9, 2047, 2048, 2055, 70001])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_reconstruct_remainders_and_alignments_agree_bitwise(gc, n, dtype):
-    # 32-byte (8 elements), 16-byte and scalar accesses by the pointers' alignment; prediction and stored x0 beside
+    # 32-byte (8 elements), 16-byte and scalar accesses by the pointers' alignment; prediction and stored x0 beside.
+    # Offsets in bytes from a 256-byte boundary: f32 buffers on 32, then 16 mod 32 with latents on 16, then one element off
     gen = torch.Generator("cuda").manual_seed(n)
     x0, xt = torch.randn(n, generator=gen, device="cuda"), torch.randn(n, generator=gen, device="cuda").to(dtype)
     outs = []
-    for off in (0, 4, 1):
-        at = lambda t, like: torch.full((n + 24,), 9.0, dtype=like.dtype, device="cuda")[off:off + n] if t is None else \
-            torch.cat([torch.zeros(off, dtype=t.dtype, device="cuda"), t])[off:]
-        a, x = at(x0, None), at(xt, None)
-        xn, pred, store = at(None, xt), at(None, x0), at(None, x0)
+    for f32_off, lat_off in ((0, 0), (16, 16), (4, x0.new_empty(0, dtype=dtype).element_size())):
+        whole = []
+
+        def at(like, fill=None):
+            off = (lat_off if like is xt else f32_off) // like.element_size()
+            buf = torch.full((n + off + 24,), 9.0, dtype=like.dtype, device="cuda")
+            whole.append((buf, off))
+            if fill is not None:
+                buf[off:off + n] = fill
+            return buf[off:off + n]
+
+        a, x = at(x0, x0), at(xt, xt)
+        xn, pred, store = at(xt), at(x0), at(x0)
         gc.reconstruct(x, a, xn, gc.make_recon("ddim", a_t=0.3, a_prev=0.4, pred_kind="eps", pred_out=pred), x0_store=store)
+        for buf, off in whole:  # nothing around the elements is written
+            assert bool((buf[:off] == 9.0).all()) and bool((buf[off + n:] == 9.0).all())
         outs.append((xn, pred, store))
     for got in outs[1:]:
         for g, r in zip(got, outs[0]):
@@ -323,17 +336,18 @@ def test_fm_velocity_and_k1(gc, workloads):
         _run_step(gc, w, g, [1, 3, 5], synth.recon_params(w, step), pred="velocity")
 
 
-@pytest.mark.parametrize("name,K,C,inplace", [("solids96", 1, 12, False), ("tiny", 4, 9, False),
-                                               ("tiny", 1, 16, True)])
-def test_plane_path_k1_and_f32(gc, workloads, name, K, C, inplace):
+@pytest.mark.parametrize("name,K,C,inplace,B", [("solids96", 1, 12, False, 4), ("tiny", 4, 9, False, 22),
+                                                 ("tiny", 1, 16, True, 1)])
+def test_plane_path_k1_and_f32(gc, workloads, name, K, C, inplace, B):
     # the increment-plane path (C >= 8) with one tap per record and with f32
     # latents: equal to the oracle, and bitwise to the record-parallel apply
-    w = workloads(name)
+    # (of enough assets that steps not in place take two launches)
+    w = synth.replicate_assets(workloads(name), B)
     g = DeviceGeometry(w, K=K, tables=False, source_index=False)
     anchors = [1, 3, 5] if w.N == 6 and w.a == 3 else [0, 3]
     params = synth.recon_params(w, 1 if w.S > 1 else 0)
-    _, _, got_plane, _ = _run_step(gc, w, g, anchors, params, C=C, inplace=inplace)
-    _, _, got_rows, _ = _run_step(gc, w, g, anchors, params, C=C, inplace=inplace, minimal_ws=True)
+    _, _, got_plane, _ = _run_step(gc, w, g, anchors, params, C=C, inplace=inplace, launches=2)
+    _, _, got_rows, _ = _run_step(gc, w, g, anchors, params, C=C, inplace=inplace, minimal_ws=True, launches=2)
     np.testing.assert_array_equal(got_plane, got_rows)
 
 
@@ -389,7 +403,8 @@ def test_random_shapes_split_the_grid_right(gc, seed):
     # random (B, N, a, C, H, W): the step kernels split their block index into
     # (asset, view, tile, channel group, record slice) with launch-invariant
     # divisors; every shape must still equal the oracle, and the sparse step
-    # the mask-mode step bit for bit (both with and without the increment plane)
+    # the mask-mode step bit for bit (both with and without the increment plane;
+    # odd seeds with as many assets as take two launches)
     rng = np.random.default_rng(9000 + seed)
     B, N = int(rng.integers(1, 4)), int(rng.integers(2, 11))
     a, C = int(rng.integers(1, N)), int(rng.integers(1, 21))
@@ -403,11 +418,15 @@ def test_random_shapes_split_the_grid_right(gc, seed):
     w = synth.Workload(**{**w.__dict__, "B": B, "N": N, "a": a, "C": C, "dtype": "bf16", "sampler": "ddim", "S": 30,
                           "cams": np.ascontiguousarray(np.tile(cams[None], (B, 1, 1))),
                           "pos": np.stack([m[0] for m in maps]), "valid": np.stack([m[1] for m in maps])})
+    if seed % 2:
+        w = synth.replicate_assets(w, max(B, 384 // (N * -(-H * W // 1024) * -(-C // 4)) + 1))
+        B = w.B
     g = DeviceGeometry(w, K=4, tables=False, source_index=False)
     anchors = sorted(rng.choice(N, size=a, replace=False).tolist())
     params = synth.recon_params(w, 7)
-    _, _, got_sparse, _ = _run_step(gc, w, g, anchors, params)
-    _, _, got_min, _ = _run_step(gc, w, g, anchors, params, minimal_ws=True)
+    launches = 2 if seed % 2 else None
+    _, _, got_sparse, _ = _run_step(gc, w, g, anchors, params, launches=launches)
+    _, _, got_min, _ = _run_step(gc, w, g, anchors, params, minimal_ws=True, launches=launches)
     _, _, got_mask, _ = _run_step(gc, w, g, anchors, params, mode="mask")
     np.testing.assert_array_equal(got_sparse, got_mask)
     np.testing.assert_array_equal(got_min, got_mask)
@@ -568,14 +587,15 @@ def test_record_overflow_is_reported_not_faulted(gc, workloads):
     assert torch.isfinite(out).all()
 
 
-@pytest.mark.parametrize("name", ["hunyuan64", "ragged"])
-def test_table_index_out_of_range_is_dropped_and_reported(gc, workloads, name):
+@pytest.mark.parametrize("H,W,B,anchors", [(64, 64, 1, [0, 3]), (37, 53, 1, [0, 3]), (32, 32, 214, [3]), (37, 29, 107, [3])])
+def test_table_index_out_of_range_is_dropped_and_reported(gc, H, W, B, anchors):
     # a caller's correspondence table with indices outside the view (past the
     # last token, and below -1): a TABLE-mode step drops those taps instead of
     # reading outside the view, reports EINVAL through the device status word,
     # and equals bit for bit the step on the same table with those taps
-    # removed (64 x 64: the staged kernel; 37 x 53: the per-tile kernel)
-    w = workloads("hunyuan64") if name == "hunyuan64" else synth.make_workload("batch128", B=1, H=37, W=53)
+    # removed (two anchors: one token per thread; large with one anchor: the
+    # staged kernel, and one CTA per tile)
+    w = synth.replicate_assets(synth.make_workload("batch128", B=2, H=H, W=W), B)
     g = DeviceGeometry(w, K=4, tables=True)
     torch.cuda.synchronize()
     HW = w.H * w.W
@@ -587,7 +607,6 @@ def test_table_index_out_of_range_is_dropped_and_reported(gc, workloads, name):
     clean_idx, clean_wt = idx.clone(), wt.clone()
     clean_idx.view(-1)[bad] = -1
     clean_wt.view(-1)[bad] = 0.0
-    anchors = [0, 3]
     x0_prev, x0_new, _ = step_inputs(w, 3, anchors)
     d_prev, d_new = torch.from_numpy(x0_prev).cuda(), torch.from_numpy(x0_new).cuda()
     outs = []
@@ -721,7 +740,7 @@ def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
     # source-tile apply (minimal workspace, corr with a source index) and the
     # record-parallel apply (minimal workspace, no index).  All three give the
     # same bits, and the oracle's results.
-    w = workloads("ring12_128") if C == 16 else workloads("solids96")
+    w = workloads("ring12_128") if C == 16 else synth.replicate_assets(workloads("solids96"), 2)
     w = synth.Workload(**{**w.__dict__, "C": C})
     g = DeviceGeometry(w, K=w.K, tables=False)
     anchors = oracle.rotate_anchors(w.N, w.a, 1)
@@ -741,6 +760,7 @@ def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
                           sigma=params.get("sigma", 0), sigma_next=params.get("sigma_next", 0))
         gc.transport_step(g.corr_for(mode), anchors, C, d_new, d_prev, d_out, d_xt, d_xn, r, workspace=ws,
                           update=update)
+        assert gc.last_launches() == 2  # two phases, not one token per thread
         torch.cuda.synchronize()
         gc.device_status()
         outs[path] = (d_out.cpu().numpy(), d_xn.cpu().view(torch.int16).numpy())
@@ -842,8 +862,9 @@ def test_wide_views_fall_back_to_the_record_parallel_apply(gc):
     pos, valid = synth.render_asset(synth.unit_sphere(), cams, H, W)
     w = synth.Workload(**{**w.__dict__, "C": 8, "cams": cams[None].astype(np.float32), "pos": pos[None],
                           "valid": valid[None]})
+    w = synth.replicate_assets(w, 2)  # 408 units: two launches
     g = DeviceGeometry(w, K=4, tables=False)
     assert g.n_records > 100
-    _, _, x0_min, _ = _run_step(gc, w, g, [0, 2, 4], synth.recon_params(w, 5), minimal_ws=True)
-    _, _, x0_plane, _ = _run_step(gc, w, g, [0, 2, 4], synth.recon_params(w, 5))
+    _, _, x0_min, _ = _run_step(gc, w, g, [0, 2, 4], synth.recon_params(w, 5), minimal_ws=True, launches=2)
+    _, _, x0_plane, _ = _run_step(gc, w, g, [0, 2, 4], synth.recon_params(w, 5), launches=2)
     np.testing.assert_array_equal(x0_min, x0_plane)

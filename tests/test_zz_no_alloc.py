@@ -44,6 +44,7 @@ def _step(gc, g, w, anchors, step, noalloc, in_place):
         gc.transport_step_noalloc(g.corr, anchors, w.C, d_new, d_prev, d_out, d_xt, d_xn, r)
     else:
         gc.transport_step(g.corr, anchors, w.C, d_new, d_prev, d_out, d_xt, d_xn, r, workspace=g.workspace(w.C))
+    assert gc.last_launches() == 2  # the steps here use the scratch
     torch.cuda.synchronize()
     gc.device_status()
     return d_out.cpu(), d_xn.cpu(), x0_prev
@@ -52,7 +53,7 @@ def _step(gc, g, w, anchors, step, noalloc, in_place):
 @pytest.mark.parametrize("in_place", [False, True])
 @pytest.mark.parametrize("sampler,lat", [("ddim", "bf16"), ("fm_euler", "bf16"), ("ddim", "f32")])
 def test_noalloc_matches_workspace_entry_point_on_consecutive_calls(gc, sampler, lat, in_place):
-    w = synth.make_workload("batch128", B=2)
+    w = synth.make_workload("batch128", B=5)  # 480 units: two launches, in place and not
     w = synth.Workload(**{**w.__dict__, "sampler": sampler, "dtype": lat, "S": 30})
     g = DeviceGeometry(w, K=4, tables=False)
     assert 0 < g.corr.workspace_floats(w.C) <= 4 * 1024 * 1024
