@@ -1761,7 +1761,8 @@ static FastDiv make_fastdiv(uint32_t d) {
 // Tile offset i of the sparse form clamped to the records that exist, [0,
 // cap]: a build whose records overflowed the capacity or the int32 offsets
 // is flagged in the status word, and the transport then reads only records
-// that exist.
+// that exist.  (An offset beyond int32 is -1, so the tile before it may end
+// before it begins: its count is taken as 0.)
 __device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_ptr, size_t i, long long cap) {
     const long long x = __ldca(tile_ptr + i);
     return (int)(x < 0 ? 0 : (x < cap ? x : cap));
@@ -1839,7 +1840,7 @@ __global__ void __launch_bounds__(kThreads, (kTokenBlocks<T, MODE>)) transport_t
                         r1 = record_offset(args.tile_ptr, i + 1, args.max_records);
                     }
                     s_r0[t] = r0;
-                    s_rn[t] = r1 - r0;
+                    s_rn[t] = max(r1 - r0, 0);
                 }
 #pragma unroll
                 for (int s2 = 0; s2 < kTokenAnchors; ++s2) s_has[s2][t] = 0;
@@ -2281,7 +2282,7 @@ __global__ void __launch_bounds__(kThreads, PK ? kPlaneBBlocks : kPhaseBBlocks<T
         // ranges clamped to the records that exist (an overflow is reported by the build)
         const int r0 = record_offset(args.tile_ptr, i, args.max_records);
         s_r0[t] = r0;
-        s_cnt[t] = record_offset(args.tile_ptr, i + 1, args.max_records) - r0;
+        s_cnt[t] = max(record_offset(args.tile_ptr, i + 1, args.max_records) - r0, 0);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {  // the sums, cleared before the wait

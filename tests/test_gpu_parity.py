@@ -587,6 +587,41 @@ def test_record_overflow_is_reported_not_faulted(gc, workloads):
     assert torch.isfinite(out).all()
 
 
+@pytest.mark.parametrize("B,C,launches", [(2, 4, 1), (40, 4, 2), (20, 16, 2)])
+def test_offsets_beyond_int32_end_the_records(gc, B, C, launches):
+    # the offsets that a build writes once its records no longer fit int32 are -1: the tile that they cut, and those
+    # after it, have no records (as if the offsets stayed where they were), whatever the kernel
+    w = synth.replicate_assets(synth.make_workload("batch128", B=2, H=64, W=64), B)
+    pos, valid, cams = (torch.from_numpy(x).cuda() for x in (w.pos, w.valid, w.cams))
+    c = gc.build_sparse_corr(pos, valid, cams)
+    ptr, rec = c._keep["tile_ptr"], c._keep["records"]
+    T, anchors = gc.tiles_per_view(w.H, w.W), [0, 3]
+    counts = (ptr[1:] - ptr[:-1]).view(B, w.N, w.N, T)
+    # cut a first tile with records of source view 0, which keeps those of source view 3 (they lie after the cut), so
+    # that a kernel that takes the cut tile's count as it comes out, negative, searches past it
+    both = (counts[:, :, 0, 0] > 0) & (counts[:, :, 3, 0] > 0)
+    both[:, anchors] = False
+    b, v = both.nonzero()[-1].tolist()
+    cut, late = (((b * w.N + v) * w.N + u) * T for u in anchors)
+    gone, stay = ptr.clone(), ptr.clone()
+    gone[cut + 1:] = -1
+    stay[cut + 1:] = ptr[cut]
+    for p in (gone, stay):
+        p[late:late + 2] = ptr[late:late + 2]
+    rnd = torch.Generator("cuda").manual_seed(2)
+    x0 = torch.randn((B, w.N, C, w.H, w.W), generator=rnd, device="cuda")
+    new = torch.randn((B, 2, C, w.H, w.W), generator=rnd, device="cuda")
+    outs = []
+    for p in (gone, stay):
+        h = gc.make_corr(pos, valid, cams, c.tau, keep=c.keep, tile_ptr=p, records=rec)
+        out = torch.empty_like(x0)
+        gc.transport_step(h, anchors, C, new, x0, out, workspace=torch.zeros(h.workspace_floats(C), device="cuda"))
+        assert gc.last_launches() == launches
+        outs.append(out)
+    gc.device_status()
+    assert torch.equal(outs[0], outs[1]) and not torch.equal(outs[0][0], x0[0])
+
+
 @pytest.mark.parametrize("H,W,B,anchors", [(64, 64, 1, [0, 3]), (37, 53, 1, [0, 3]), (32, 32, 214, [3]), (37, 29, 107, [3])])
 def test_table_index_out_of_range_is_dropped_and_reported(gc, H, W, B, anchors):
     # a caller's correspondence table with indices outside the view (past the
