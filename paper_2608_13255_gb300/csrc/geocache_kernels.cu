@@ -1278,9 +1278,10 @@ __device__ __forceinline__ uint32_t quad_masks(const uint8_t* row, int cnt, bool
 //    compacted into a work list (block prefix sum, token order) and processed one
 //    per thread, so the dependent loads of many tokens overlap (MASK: keep masks
 //    -> target position -> projection and weights -> gathers of the anchor
-//    increments x0_new - x0(t-1) at the kept taps).  Per-anchor sums are combined in anchor order (Eq. 1 with the
-//    multi-anchor aggregation of Sec. 3.2: the mean over covering anchors; a
-//    token without a kept tap keeps x0(t-1)).
+//    increments x0_new - x0(t-1) at the kept taps).  Per-anchor sums are
+//    combined in anchor order (Eq. 1 with the multi-anchor aggregation of Sec.
+//    3.2: the mean over covering anchors; a token without a kept tap keeps
+//    x0(t-1)).
 //  * Every token is stored (x0(t)) and reconstructed (x_{t-1}) from the
 //    staged rows with 16-byte stores.
 constexpr int kTileTokens = 4 * kThreads;
@@ -1768,8 +1769,9 @@ __device__ __forceinline__ int record_offset(const int32_t* __restrict__ tile_pt
     return (int)(x < 0 ? 0 : (x < cap ? x : cap));
 }
 
-// Most TABLE and GEOMETRY steps, and MASK and SPARSE steps of few units: one CTA per 256 tokens
-// of a view and group of 4 channels, one token per thread, any alignment.
+// Most TABLE and GEOMETRY steps, and MASK and SPARSE steps of few units: one CTA
+// per 256 tokens of a view and group of 4 channels, one token per thread, any
+// alignment.
 // The two kernels above take a tile of 1024 tokens per CTA, whose work items
 // (token, anchor; up to 4 per token and round of anchors) go 256 at a time
 // through a chain of dependent loads with a barrier per anchor; where their
