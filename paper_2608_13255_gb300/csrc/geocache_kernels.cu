@@ -2454,15 +2454,16 @@ __global__ void __launch_bounds__(kThreads, kPlaneABlocks) sparse_phase_a_plane_
 // x0_new - x0(t-1) (x0_new itself for the value copy) of the tile and of the
 // W + 1 tokens after it in shared memory ([token][4 channels]: every tap of a
 // record whose first kept tap lies in the tile), streams the anchor tile
-// itself (x0(t) and the reconstruction) unless the update is in place, and
-// then applies the tile's group of the source index: for each record whose
-// target view is outside the anchor set, sum_k w_k increment[q_k] in tap
-// order, read from shared memory, into its workspace row.  The scattered
-// per-channel gathers of the record-parallel apply become one coalesced read
-// of the anchor tile.
+// itself (x0(t) and the reconstruction) unless the update is in place (both in
+// 16-byte words with vec_rows, where every row starts on one), and then applies
+// the tile's group of the source index: for each record whose target view is
+// outside the anchor set, sum_k w_k increment[q_k] in tap order, read from
+// shared memory, into its workspace row.  The scattered per-channel gathers of
+// the record-parallel apply become one coalesced read of the anchor tile.
 template <typename T, int K, bool COPY>
 __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_src_kernel(const TransportArgs args,
-                                                                                       const SparseGrid g, int stream) {
+                                                                                       const SparseGrid g, bool stream,
+                                                                                       bool vec_rows) {
     pdl_launch_dependents();
     extern __shared__ __align__(16) float4 s_d[];  // [kTileTokens + W + 1] tokens x 4 channels
     const int HW = args.H * args.W, W = args.W;
@@ -2484,7 +2485,6 @@ __global__ void __launch_bounds__(kThreads, kPhaseABlocks<T>) sparse_phase_a_src
     const size_t view_base = ((size_t)b * N + u) * C * plane;
     const T* xt_p = static_cast<const T*>(args.x_t);
     T* xn_p = static_cast<T*>(args.x_next);
-    const bool vec_rows = (HW & 3) == 0;
     for (int q = threadIdx.x; 4 * q < span; q += kThreads) {
         const int p0 = tile0 + 4 * q;
         const int cnt = min(4, span - 4 * q);
@@ -2646,9 +2646,9 @@ static cudaError_t launch_sparse(const TransportArgs& t, cudaStream_t s) {
         if (g > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         const size_t dyn = (size_t)(kTileTokens + t.W + 1) * sizeof(float4);
         if (!copy)
-            sparse_phase_a_src_kernel<T, K, false><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
+            sparse_phase_a_src_kernel<T, K, false><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, !in_place, vec);
         else
-            sparse_phase_a_src_kernel<T, K, true><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, in_place ? 0 : 1);
+            sparse_phase_a_src_kernel<T, K, true><<<(unsigned)g, kThreads, dyn, s>>>(t, sg, !in_place, vec);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         phase_a = true;

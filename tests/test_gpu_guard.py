@@ -87,16 +87,19 @@ def _geometry(gc, w, K=4, skew=0, records_frac=1.0):
     ("ragged_c5", 2, 2), ("ragged_c5", 20, 2),    # one token per thread; beside it two launches, masks by tile
     ("ragged_c18", 2, 2), ("ragged_c18", 9, 2), ("ragged_c18_src", 9, 2), ("ragged_c18_src", 2, 2),
     ("misaligned", 1, 2), ("misaligned", 22, 2),
+    ("misaligned_src", 1, 2), ("misaligned_src", 22, 2),
     ("c3_k1", 1, 2), ("c3_k1", 110, 1),           # masks and geometry by tile from staged rows
     ("aligned_c6", 22, 3)])
 def test_transport_writes_only_its_outputs(gc, case, B, a):
-    minimal_ws = case == "ragged_c18_src"  # the source-tile apply instead of the increment plane
+    minimal_ws = case.endswith("_src")  # the source-tile apply instead of the increment plane
     if case == "ragged_c5":  # 37 x 53 tokens: H*W = 1961, two tiles, a ragged quad; C = 5
         w, C, skew, K = synth.make_workload("batch128", B=2, H=37, W=53), 5, 0, 4
     elif case in ("ragged_c18", "ragged_c18_src"):  # the same with C = 18: a partial last channel group
         w, C, skew, K = synth.make_workload("batch128", B=2, H=37, W=53), 18, 0, 4
     elif case == "misaligned":  # 64 x 64 tokens, every buffer 4 bytes off a 16-byte boundary
         w, C, skew, K = synth.make_workload("hunyuan64"), 4, 4, 4
+    elif case == "misaligned_src":  # the same with C = 10
+        w, C, skew, K = synth.make_workload("hunyuan64"), 10, 4, 4
     elif case == "aligned_c6":  # 64 x 64 tokens, 16-byte words
         w, C, skew, K = synth.make_workload("batch128", B=2, H=64, W=64), 6, 0, 4
     else:

@@ -767,14 +767,16 @@ def test_source_index_groups_every_record_once(gc, workloads, name):
     np.testing.assert_array_equal(ent[order, 1], v)
 
 
-@pytest.mark.parametrize("C,update,inplace", [(16, "delta", False), (16, "delta", True), (20, "copy", False),
-                                              (33, "delta", False), (8, "copy", True)])
-def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
+@pytest.mark.parametrize("C,update,inplace,off", [(16, "delta", False, 0), (16, "delta", True, 0), (20, "copy", False, 0),
+                                                  (33, "delta", False, 0), (8, "copy", True, 0),
+                                                  (20, "delta", False, 1), (9, "copy", True, 3)])
+def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace, off):
     # wide latents (C >= 8) have three ways to form the records' increments:
     # the anchors' increment plane (workspace with room for it), the
     # source-tile apply (minimal workspace, corr with a source index) and the
     # record-parallel apply (minimal workspace, no index).  All three give the
-    # same bits, and the oracle's results.
+    # same bits, and the oracle's results (off: buffers that many elements off
+    # their alignment, of views whose rows are a multiple of 16 bytes).
     w = workloads("ring12_128") if C == 16 else synth.replicate_assets(workloads("solids96"), 2)
     w = synth.Workload(**{**w.__dict__, "C": C})
     g = DeviceGeometry(w, K=w.K, tables=False)
@@ -788,9 +790,13 @@ def test_wide_latent_paths_agree_bitwise(gc, workloads, C, update, inplace):
             assert ws.numel() >= g.corr.min_workspace_floats(C) + len(anchors) * w.B * -(-C // 4) * 4 * w.H * w.W
         x0_prev, x0_new, xt32 = step_inputs(w, 3, anchors)
         xt64, xt = latent_values(xt32, w)
-        d_prev, d_new, d_xt = torch.from_numpy(x0_prev).cuda(), torch.from_numpy(x0_new).cuda(), xt.cuda()
-        d_out = d_prev if inplace else torch.empty_like(d_prev)
-        d_xn = d_xt if inplace else torch.empty_like(d_xt)
+        def at(t):
+            buf = torch.empty(t.numel() + off, dtype=t.dtype, device="cuda")[off:].view(t.shape)
+            return buf.copy_(t)
+
+        d_prev, d_new, d_xt = at(torch.from_numpy(x0_prev)), at(torch.from_numpy(x0_new)), at(xt)
+        d_out = d_prev if inplace else at(d_prev)
+        d_xn = d_xt if inplace else at(d_xt)
         r = gc.make_recon(params["sampler"], a_t=params.get("a_t", 0), a_prev=params.get("a_prev", 0),
                           sigma=params.get("sigma", 0), sigma_next=params.get("sigma_next", 0))
         gc.transport_step(g.corr_for(mode), anchors, C, d_new, d_prev, d_out, d_xt, d_xn, r, workspace=ws,
