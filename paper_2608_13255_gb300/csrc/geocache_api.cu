@@ -305,6 +305,7 @@ int geocache_transport_step_update(const geocache_corr* c, geocache_update updat
             return fail(GEOCACHE_EINVAL, "sparse mode needs a workspace of max_records * C = %lld floats",
                         (long long)(c->max_records * (int64_t)C));
         if (((uintptr_t)workspace & 15)) return fail(GEOCACHE_EINVAL, "workspace must be 16-byte aligned");
+        if (c->src_ptr && ((uintptr_t)c->src_rec & 7)) return fail(GEOCACHE_EINVAL, "src_rec must be 8-byte aligned");
     } else {
         return fail(GEOCACHE_EINVAL, "unknown corr mode %d", (int)c->mode);
     }

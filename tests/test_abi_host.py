@@ -121,6 +121,11 @@ def test_argument_errors_before_launch(gc):
                                    None, None, 0, None, None, 0, None)
     assert st == gc.EINVAL and "workspace" in gc.last_error()
     assert L.geocache_transport_workspace(ctypes.byref(c), 4) == 40
+    c.src_ptr, c.src_rec = 64, 132  # the source index' entries are read as 8-byte words
+    st = L.geocache_transport_step(ctypes.byref(c), ctypes.cast(anc, ctypes.c_void_p), 2, 4, 16, 16, 32,
+                                   None, None, 0, None, 4096, 40, None)
+    assert st == gc.EINVAL and "src_rec" in gc.last_error()
+    c.src_ptr = c.src_rec = None
     c.tile_ptr, c.records, c.max_records = None, None, 0
     c.mode = gc.CORR_GEOMETRY
     assert L.geocache_transport_workspace(ctypes.byref(c), 4) == 0
